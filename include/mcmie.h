@@ -288,12 +288,12 @@ mc_status mc_run_static(const mc_medium *medium, const mc_geometry *geom,
                         int64_t *d_image, int64_t *d_radial, int64_t *d_totals,
                         uint32_t *d_error, void *stream);
 
-/* Many media in one launch: every CTA goes through the media in order of
- * decreasing estimated cost (photons x (1 + optical depth along x)); its warps
- * take chunks of item_photons photons of the current medium from that
- * medium's counter (0: 128; else 32 .. 2^20), and when the medium's photons
- * are all taken the CTA flushes its tallies into the medium's, stages the
- * next medium's table in shared memory and goes on, so the media follow one
+/* Many media in one launch: the CTAs are shared out among the media by
+ * estimated photon-steps; a CTA's warps take chunks of item_photons photons
+ * of its medium from that medium's counter (0: 128; else 32 .. 2^20), and
+ * when the medium's photons are all taken the CTA flushes its tallies into
+ * the medium's, joins the medium with most work left per CTA (staging its
+ * table in shared memory) and goes on, so the media follow one
  * another without launch gaps. All instances share geometry, camera and run
  * parameters (run->n_photons, photon_offset and seed are ignored; each
  * instance has its own), and one phase kind and table size. Tallies per

@@ -388,47 +388,29 @@ mc_status mc_run_batch(int n, const mc_instance *inst, const mc_geometry *geom, 
         if ((e = mcx::check_plan(c, launch_cfg(run))) != cudaSuccess)
             return e == cudaErrorInvalidValue ? MC_ERR_ARG : MC_ERR_CUDA;
     }
-    if (!run->accumulate)
-        for (int i = 0; i < n; ++i) {
-            if ((e = cudaMemsetAsync(inst[i].d_image, 0, sizeof(int64_t) * (size_t)camera->nx * camera->nz, st)) ||
-                (e = cudaMemsetAsync(inst[i].d_radial, 0, sizeof(int64_t) * (size_t)camera->n_radial, st)) ||
-                (e = cudaMemsetAsync(inst[i].d_totals, 0, sizeof(int64_t) * MC_N_TOTALS, st)))
-                return MC_ERR_CUDA;
-        }
-    if ((e = cudaMemsetAsync(d_work, 0, sizeof(unsigned long long) * (size_t)n, st))) return MC_ERR_CUDA;
-
-    // largest estimated cost first: photons x (1 + optical depth along the beam)
-    int order[mcx::kMaxBatch];
-    double cost[mcx::kMaxBatch];
-    for (int i = 0; i < n; ++i) {
-        order[i] = i;
-        cost[i] = (double)inst[i].n_photons * (1.0 + (inst[i].medium.mu_s + inst[i].medium.mu_a) * geom->lx);
-    }
-    for (int i = 1; i < n; ++i)   // stable insertion sort, descending
-        for (int j = i; j > 0 && cost[order[j]] > cost[order[j - 1]]; --j) {
-            int t = order[j]; order[j] = order[j - 1]; order[j - 1] = t;
-        }
     mcx::BatchArgs *a = new (std::nothrow) mcx::BatchArgs;
     if (!a) return MC_ERR_NOMEM;
     std::memset(a, 0, sizeof *a);
-    uint64_t n_max = 0, n_all = 0;
-    for (int i = 0; i < n; ++i) {
-        n_max = inst[i].n_photons > n_max ? inst[i].n_photons : n_max;
-        n_all += inst[i].n_photons;
-    }
+    uint64_t n_max = 0;
+    for (int i = 0; i < n; ++i) n_max = inst[i].n_photons > n_max ? inst[i].n_photons : n_max;
     fill_common(a->c, &inst[0].medium, geom, camera, run, d_error, n_max);
     a->n_media = n;
     a->chunk = item_photons ? (unsigned)item_photons : 128u;
     a->counters = static_cast<unsigned long long *>(d_work);
-    for (int k = 0; k < n; ++k) {
-        const mc_instance &I = inst[order[k]];
-        fill_medium(a->m[k], &I.medium, I.n_photons, I.photon_offset, I.seed, I.d_image, I.d_radial, I.d_totals);
+    double total = 0.0, sum = 0.0;
+    for (int i = 0; i < n; ++i) {
+        const mc_instance &I = inst[i];
+        fill_medium(a->m[i], &I.medium, I.n_photons, I.photon_offset, I.seed, I.d_image, I.d_radial, I.d_totals);
+        // 1.9 steps per photon at optical depth 1 along the beam, 4.3 at 5,
+        // 8.8 at 20 (4.5:1 cuvette); only the CTAs' shares depend on it
+        a->steps[i] = (float)(1.0 + 1.2 * std::pow((I.medium.mu_s + I.medium.mu_a) * geom->lx, 0.62));
+        total += (double)I.n_photons * a->steps[i];
     }
-    if (n_all == 0) {
-        delete a;
-        return MC_OK;
+    for (int i = 0; i < n; ++i) {
+        sum += (double)inst[i].n_photons * a->steps[i];
+        a->share[i] = total > 0.0 ? (float)(sum / total) : 0.0f;
     }
-    e = mcx::launch_batch(*a, launch_cfg(run), st);
+    e = mcx::launch_batch(*a, !run->accumulate, launch_cfg(run), st);
     delete a;
     return cuda_status(e);
 }

@@ -56,14 +56,16 @@ struct WalkArgs {
     unsigned long long *counter;  // photon counter in the caller's workspace
 };
 
-// Many media in one launch, processed in the order of m[]: medium i's photons
-// are taken in warp chunks of `chunk` from counters[i] (caller's workspace).
+// Many media in one launch: medium i's photons are taken in warp chunks of
+// `chunk` from counters[i] (caller's workspace).
 constexpr int kMaxBatch = 64;
 struct BatchArgs {
     CommonArgs c;
     int n_media;
     unsigned chunk;               // photons a warp takes from a counter at once (>= 32)
-    unsigned long long *counters; // [n_media] photon counters
+    unsigned long long *counters; // [n_media] photon counters (and the CTAs on each medium)
+    float steps[kMaxBatch];       // estimated photon-steps per photon
+    float share[kMaxBatch];       // running sum of estimated photon-steps up to and with medium i, as a fraction
     MediumArgs m[kMaxBatch];
 };
 
@@ -141,8 +143,9 @@ cudaError_t launch_walk(const WalkArgs &a, bool trace, const LaunchCfg &cfg, cud
 // do not fit in one CTA's shared memory.
 cudaError_t check_plan(const CommonArgs &c, const LaunchCfg &cfg);
 
-// Launch the batched walk (phase fixed by c.phase_kind) on `stream`.
-cudaError_t launch_batch(const BatchArgs &a, const LaunchCfg &cfg, cudaStream_t stream);
+// Launch the batched walk (phase fixed by c.phase_kind) on `stream`, after
+// clearing the counters and, when fresh, the media's tallies.
+cudaError_t launch_batch(const BatchArgs &a, bool fresh, const LaunchCfg &cfg, cudaStream_t stream);
 
 // Launch the adjoint replay and the reduction into out[3 + n_w]
 // (value, dL/dmu_s, dL/dmu_a, dL/dw_k). partial_rows: capacity of partials.

@@ -781,15 +781,47 @@ __global__ void __launch_bounds__(1024) walk_kernel(const __grid_constant__ Walk
     flush<SMEM_IMAGE>(A.c, A.m, S, T);
 }
 
-// Many media in one launch: every CTA goes through the media in the order
-// given (largest estimated cost first). Its warps take chunks of the current
-// medium's photons from that medium's global counter, as in the one-medium
-// launch; once the counter is exhausted and the CTA's warps have finished
-// their photons, the CTA flushes its tallies into the medium's, stages the
-// next medium's table and goes on. CTAs flow from one medium into the next
-// without launch gaps, every medium's photons spread over all CTAs at warp-
-// chunk granularity; a CTA skips a medium whose photons were all taken
-// before it arrived.
+// A batch counter holds the medium's next photon in its low bits and the
+// CTAs that joined the medium above them.
+constexpr unsigned long long JOIN = 1ull << 40;
+constexpr float JOIN_STEPS = 8192.f;   // photon-steps per CTA below which joining a running medium does not pay
+
+// The medium a CTA works on next (warp 0, all lanes): the one with most
+// estimated photon-steps left per CTA on it, and any medium that no CTA has
+// joined yet; -1 when neither is left. Called again and again, so every
+// medium is joined: a CTA leaves only after seeing none without CTAs.
+__device__ __forceinline__ int pick_medium(const BatchArgs &B, int lane)
+{
+    float best = 0.f;
+    int at = -1;
+    for (int m = lane; m < B.n_media; m += 32) {
+        const unsigned long long c = *reinterpret_cast<volatile unsigned long long *>(B.counters + m);
+        const unsigned long long next = c & (JOIN - 1), n = B.m[m].n_photons;
+        if (next >= n) continue;
+        const unsigned workers = (unsigned)(c >> 40);
+        const float left = (float)(n - next) * B.steps[m] / (float)(workers + 1);
+        if (workers && left < JOIN_STEPS) continue;
+        if (at < 0 || left > best) { best = left; at = m; }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const float b2 = __shfl_xor_sync(FULL, best, o);
+        const int a2 = __shfl_xor_sync(FULL, at, o);
+        if (a2 >= 0 && (at < 0 || b2 > best || (b2 == best && a2 < at))) { best = b2; at = a2; }
+    }
+    return at;
+}
+
+// Many media in one launch, the CTAs shared out among them: CTA b starts on
+// the medium where the running sum of estimated photon-steps passes the
+// fraction (b + 1/2) / CTAs, and its warps take chunks of that medium's
+// photons from the medium's counter, as in the one-medium launch. Once the
+// counter is exhausted and the CTA's warps have finished their photons, the
+// CTA flushes its tallies into the medium's and joins the medium with most
+// work left per CTA. A CTA thus stages few tables and flushes few images, and
+// one medium's drain overlaps other media's work: 64 media of 2e5 photons on
+// 128 x 128 images take 0.85 ms a call against 3.87 ms when every CTA went
+// through every medium (the grid then was as large as the largest medium
+// could feed, 49 CTAs); 64 media of 1e6 to 1e8 photons 78.8 against 83.2 ms.
 template <int PHASE, bool SMEM_IMAGE>
 __global__ void __launch_bounds__(1024) batch_kernel(const __grid_constant__ BatchArgs B)
 {
@@ -801,16 +833,31 @@ __global__ void __launch_bounds__(1024) batch_kernel(const __grid_constant__ Bat
     Tally T{0u, 0ll, 0ll, 0ll, 0ll, 0ll};
     uint32_t parity = 0;
     const unsigned chunk = B.chunk;
-    for (int m = 0; m < B.n_media; ++m) {
+    for (bool first = true;; first = false) {
+        if (threadIdx.x < 32) {
+            int m = -1;
+            if (first) {
+                const float mine = ((float)blockIdx.x + 0.5f) / (float)gridDim.x;
+                m = 0;
+                while (m < B.n_media - 1 && B.share[m] <= mine) ++m;
+                const unsigned long long next =
+                    *reinterpret_cast<volatile unsigned long long *>(B.counters + m) & (JOIN - 1);
+                if (next >= B.m[m].n_photons) m = -1;
+            }
+            if (m < 0) m = pick_medium(B, threadIdx.x);
+            if (threadIdx.x == 0) {
+                if (m >= 0) atomicAdd(B.counters + m, JOIN);
+                *S.item = (unsigned long long)(long long)m;
+            }
+        }
+        __syncthreads();
+        const int m = (int)(long long)*S.item;
+        __syncthreads();
+        if (m < 0) break;
         // this medium's arguments, copied once: read through the dynamically
         // indexed kernel parameter, every use in the walk would be a load
         const MediumArgs M = B.m[m];
         unsigned long long *ctr = B.counters + m;
-        if (threadIdx.x == 0) *S.item = *reinterpret_cast<volatile unsigned long long *>(ctr);
-        __syncthreads();
-        const bool taken = *S.item >= M.n_photons;
-        __syncthreads();
-        if (taken) continue;
         if (PHASE != MC_PHASE_HG) {
             if (!stage_bulk(S.table, M.table, B.c.table_bytes, S.bar, parity, B.c.error)) return;
             parity ^= 1u;
@@ -821,14 +868,27 @@ __global__ void __launch_bounds__(1024) batch_kernel(const __grid_constant__ Bat
 #pragma unroll
         for (int i = 0; i < 20; ++i) rk[i] = M.rk[i];
         walk_loop<PHASE, SMEM_IMAGE, false>(
-            B.c, M, rk, S, M.n_photons, chunk, [ctr, chunk]() { return atomicAdd(ctr, (unsigned long long)chunk); },
-            T);
+            B.c, M, rk, S, M.n_photons, chunk,
+            [ctr, chunk]() { return atomicAdd(ctr, (unsigned long long)chunk) & (JOIN - 1); }, T);
         flush<SMEM_IMAGE>(B.c, M, S, T);
         zero_tallies(S, B.c);
         __syncthreads();
     }
 }
 
+// Fresh tallies and photon counters of a batch: blocks of medium blockIdx.y
+// clear its image, radial profile, totals and counter.
+constexpr int ZERO_BLOCK = 256;
+__global__ void __launch_bounds__(ZERO_BLOCK) batch_zero_kernel(const __grid_constant__ BatchArgs B, bool tallies)
+{
+    const MediumArgs &M = B.m[blockIdx.y];
+    const int t = blockIdx.x * ZERO_BLOCK + threadIdx.x, nt = gridDim.x * ZERO_BLOCK;
+    if (t == 0) B.counters[blockIdx.y] = 0ull;
+    if (!tallies) return;
+    for (int i = t; i < B.c.nx * B.c.nz; i += nt) M.image[i] = 0ull;
+    for (int i = t; i < B.c.n_radial; i += nt) M.radial[i] = 0ull;
+    if (t < MC_N_TOTALS) M.totals[t] = 0ull;
+}
 
 // ------------------------------------------------------- heterogeneous medium
 // Delta (Woodcock) tracking through a voxel grid (the complex media of
@@ -2023,11 +2083,8 @@ cudaError_t launch_batch_one(const BatchArgs &a, const LaunchCfg &cfg, size_t sm
 {
     auto kern = batch_kernel<PHASE, SMEM_IMAGE>;
     unsigned grid = 0;
-    unsigned long long chunks = 0;   // warp chunks of the largest medium: more warps would idle
-    for (int i = 0; i < a.n_media; ++i) {
-        const unsigned long long c = (a.m[i].n_photons + a.chunk - 1) / a.chunk;
-        if (c > chunks) chunks = c;
-    }
+    unsigned long long chunks = 0;   // warp chunks of all media: more warps would idle
+    for (int i = 0; i < a.n_media; ++i) chunks += (a.m[i].n_photons + a.chunk - 1) / a.chunk;
     cudaError_t e = launch_persistent(kern, &a, cfg, smem, chunks, &grid);
     if (e != cudaSuccess) return e;
     kern<<<grid, cfg.block, smem, st>>>(a);
@@ -2196,7 +2253,7 @@ cudaError_t launch_grid_adjoint(const GridAdjArgs &a, int rows, double *value, c
     }
 }
 
-cudaError_t launch_batch(const BatchArgs &a0, const LaunchCfg &cfg0, cudaStream_t st)
+cudaError_t launch_batch(const BatchArgs &a0, bool fresh, const LaunchCfg &cfg0, cudaStream_t st)
 {
     BatchArgs a = a0;
     LaunchCfg cfg = cfg0;
@@ -2204,6 +2261,10 @@ cudaError_t launch_batch(const BatchArgs &a0, const LaunchCfg &cfg0, cudaStream_
     size_t smem = 0;
     cudaError_t e = plan_image(a.c, cfg, &smem_img, &smem);
     if (e != cudaSuccess) return e;
+    bool any = false;
+    for (int i = 0; i < a.n_media; ++i) any |= a.m[i].n_photons != 0;
+    batch_zero_kernel<<<dim3(fresh ? sign_blocks(a.c) : 1, (unsigned)a.n_media), ZERO_BLOCK, 0, st>>>(a, fresh);
+    if ((e = cudaGetLastError()) != cudaSuccess || !any) return e;
     switch (a.c.phase_kind * 2 + (smem_img ? 1 : 0)) {
     case 0: e = launch_batch_one<MC_PHASE_TABLE, false>(a, cfg, smem, st); break;
     case 1: e = launch_batch_one<MC_PHASE_TABLE, true>(a, cfg, smem, st); break;
