@@ -152,6 +152,11 @@ void fill_common(mcx::CommonArgs &c, const mc_medium *m, const mc_geometry *g, c
     c.phase_kind = m->phase_kind;
     c.table_bytes = (uint32_t)table_bytes_of(m);
     c.n_bins = (m->phase_kind != MC_PHASE_HG) ? m->n_bins : 0;
+    c.log2_bins = 0;
+    if (m->phase_kind == MC_PHASE_TABLE)
+        while ((1 << c.log2_bins) < m->n_bins) ++c.log2_bins;
+    c.bin_shift = 23 - c.log2_bins;
+    c.frac_one = (float)(1.0 - std::ldexp(1.0, c.log2_bins - 24));
     c.lx = (float)g->lx;
     c.hy = (float)(0.5 * g->ly);
     c.hz = (float)(0.5 * g->lz);

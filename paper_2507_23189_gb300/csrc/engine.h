@@ -29,6 +29,11 @@ struct CommonArgs {
     int phase_kind;             // MC_PHASE_TABLE / MC_PHASE_HG (one per launch)
     uint32_t table_bytes;
     int n_bins;
+    // an inverse-CDF table's n_bins = 2^log2_bins: a 23-bit uniform's bin is
+    // its bits from bin_shift = 23 - log2_bins up, its fraction a mantissa
+    // minus frac_one = 1 - 2^(log2_bins - 24)
+    int log2_bins, bin_shift;
+    float frac_one;
     // geometry
     float lx, hy, hz, beam_r;
     // camera
