@@ -400,7 +400,7 @@ mc_status mc_run_batch(int n, const mc_instance *inst, const mc_geometry *geom, 
     for (int i = 0; i < n; ++i) n_max = inst[i].n_photons > n_max ? inst[i].n_photons : n_max;
     fill_common(a->c, &inst[0].medium, geom, camera, run, d_error, n_max);
     a->n_media = n;
-    a->chunk = item_photons ? (unsigned)item_photons : 128u;
+    a->max_per = item_photons ? (unsigned)(item_photons / 32) : 4u;
     a->counters = static_cast<unsigned long long *>(d_work);
     double total = 0.0, sum = 0.0;
     for (int i = 0; i < n; ++i) {

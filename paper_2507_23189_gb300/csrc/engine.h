@@ -61,13 +61,13 @@ struct WalkArgs {
     unsigned long long *counter;  // photon counter in the caller's workspace
 };
 
-// Many media in one launch: medium i's photons are taken in warp chunks of
-// `chunk` from counters[i] (caller's workspace).
+// Many media in one launch: warps take medium i's photons from counters[i]
+// (caller's workspace).
 constexpr int kMaxBatch = 64;
 struct BatchArgs {
     CommonArgs c;
     int n_media;
-    unsigned chunk;               // photons a warp takes from a counter at once (>= 32)
+    unsigned max_per;             // 32 max_per: photons a warp takes from a counter at once, at most
     unsigned long long *counters; // [n_media] photon counters (and the CTAs on each medium)
     float steps[kMaxBatch];       // estimated photon-steps per photon
     float share[kMaxBatch];       // running sum of estimated photon-steps up to and with medium i, as a fraction

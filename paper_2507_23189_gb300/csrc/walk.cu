@@ -26,7 +26,6 @@ namespace mcx {
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr int CHUNK = 128;            // photons a warp takes from the counter at once
 constexpr float INV_2PI = 0.159154943091895335768883763372514f;
 constexpr float W_SCALE = 4294967296.0f;   // 2^32, weight tallies
 constexpr uint32_t WAIT_LIMIT = 1u << 22;  // mbarrier polls before giving up
@@ -297,14 +296,14 @@ __device__ __forceinline__ void trace_write(const CommonArgs &C, unsigned long l
 }
 
 // Shared memory of a walk CTA:
-//   [table blob][image band][radial][totals][mbarrier][item][pool]
+//   [table blob][image band][radial][totals][mbarrier][item, 2 words]
 // and the views of the staged table: omu / pdf / guide of the inverse-CDF
 // table, or, for the paper's table, omu (node 1 - cos theta), pdf (density
 // per radian), pk / pdl / pri (search thresholds and interpolation aids).
 struct Smem {
     unsigned char *table;
     uint32_t *img;            // low 32 bits of the privatised image pixels
-    unsigned long long *rad, *tot, *bar, *item, *pool;
+    unsigned long long *rad, *tot, *bar, *item;   // item: 2 words
     int npix;                 // privatised image pixels (band rows x nx)
     const float *omu, *pdf;
     const uint16_t *guide;
@@ -495,7 +494,6 @@ __device__ __forceinline__ Smem carve(unsigned char *smem, const CommonArgs &C)
     S.tot = S.rad + C.n_radial;
     S.bar = S.tot + MC_N_TOTALS;
     S.item = S.bar + 1;
-    S.pool = S.item + 1;
     S.omu = S.pdf = S.pdl = S.pri = nullptr;
     S.guide = nullptr;
     S.pk = nullptr;
@@ -587,75 +585,152 @@ __device__ void flush(const CommonArgs &C, const MediumArgs &M, const Smem &S, T
     __syncthreads();
 }
 
-// The photon walk over indices [.., limit) of medium M: every warp refills
-// lanes whose photon ended from chunks of `chunk` indices obtained by
-// grab() (called by lane 0), until the range is exhausted.
-// rk: the Philox round keys of M's seed (M.rk, or a copy of them).
-template <int PHASE, bool SMEM_IMAGE, bool TRACE, class Grab>
-__device__ __forceinline__ void walk_loop(const CommonArgs &C, const MediumArgs &M, const uint32_t (&rk)[20],
-                                          const Smem &S, unsigned long long limit, unsigned chunk, Grab grab,
-                                          Tally &T)
+// A warp's photons: its lanes take them one at a time from the warp's pool,
+// and a warp whose pool is used up takes 32 per photons from the range's
+// counter. per falls with what was left of the range when the warp last looked
+// (half of what each lane would get from an even split, MAX_PER at most), so
+// that all warps end together: against fixed chunks of 128 photons from the
+// counter and 64-bit pools, 20 000 photons on a 64 x 64 image take 24 us a call
+// instead of 36 (the CTAs spread over all SMs, too), a delta-tracking image and
+// gradient of 5e5 photons 1.14 ms instead of 1.32, 1e8 photons at tau 5 1.7 %
+// less. (Lanes that own shares of up to 16 photons skip the ballot at most
+// ends, but at 20 to 60 photons per lane that is up to 22 % slower: lanes end
+// their last shares alone.)
+constexpr uint32_t MAX_PER = 4;
+
+// A launch's range [0, limit): warps get their first 32 per photons by their
+// number (interleaved over the CTAs, so that a small range is spread over all
+// SMs), the rest from the counter, which starts at 0. What the formulas need
+// is recomputed at each grab, to keep it out of the walk's registers.
+struct LaunchRange {
+    unsigned long long *counter;
+    uint32_t limit;             // photons, at most 2^31
+    __device__ __forceinline__ uint32_t warps() const { return gridDim.x * (blockDim.x >> 5); }
+    __device__ __forceinline__ uint32_t per(uint32_t seen) const
+    {
+        return min(max((uint32_t)((float)(limit - seen) * (0.015625f / (float)warps())), 1u), MAX_PER);
+    }
+    __device__ __forceinline__ unsigned long long first(uint32_t warp) const
+    {
+        return (unsigned long long)warp * (32u * per(0u));
+    }
+    __device__ __forceinline__ unsigned long long grab(uint32_t n) const   // one lane
+    {
+        const unsigned long long given = first(warps());
+        return given >= limit ? given : given + atomicAdd(counter, (unsigned long long)n);
+    }
+};
+
+// A batch counter holds the medium's next photon in its low bits and the
+// CTAs that joined the medium above them.
+constexpr unsigned long long JOIN = 1ull << 40;
+
+// One medium of a batch: the counter's low bits; lanes: those on the medium
+// when the CTA joined it.
+struct BatchRange {
+    unsigned long long *counter;
+    uint32_t limit, max_per;
+    float inv_share;            // 1 / (2 lanes)
+    __device__ __forceinline__ uint32_t per(uint32_t seen) const
+    {
+        return min(max((uint32_t)((float)(limit - seen) * inv_share), 1u), max_per);
+    }
+    __device__ __forceinline__ unsigned long long grab(uint32_t n) const   // one lane
+    {
+        return atomicAdd(counter, (unsigned long long)n) & (JOIN - 1);
+    }
+};
+
+struct Pool {                                // all warp-uniform
+    uint32_t next = 0, end = 0;              // the warp's photons not yet started
+    uint32_t seen = 0;                       // photons given out when the warp last looked
+    bool dry = false;                        // the range is used up
+
+    // The next photon of each lane in `need` (the limit or beyond: none). The
+    // whole warp calls it.
+    template <class Range>
+    __device__ __forceinline__ uint32_t take(const Range &R, unsigned need)
+    {
+        const int lane = threadIdx.x & 31;
+        const uint32_t n = __popc(need), rank = __popc(need & ((1u << lane) - 1u)), avail = end - next;
+        if (avail >= n) {
+            next += n;
+            return next - n + rank;
+        }
+        uint32_t base = R.limit;
+        const uint32_t first = next;
+        if (!dry) {
+            const uint32_t take = 32u * R.per(seen);
+            unsigned long long b = 0;
+            if (lane == 0) b = min(R.grab(take), (unsigned long long)R.limit);
+            seen = base = __shfl_sync(FULL, (uint32_t)b, 0);
+            dry = base >= R.limit;
+            next = base + (n - avail);
+            end = base + take;
+        } else {
+            next = end = base;
+        }
+        return rank < avail ? first + rank : base + (rank - avail);
+    }
+};
+
+__device__ __forceinline__ Pool launch_pool(const LaunchRange &R)
 {
-    const int lane = threadIdx.x & 31;
-    const unsigned lanemask_lt = (1u << lane) - 1u;
-    unsigned long long pool_next = 0, pool_end = 0;  // warp-uniform
+    Pool p;
+    const unsigned long long base = R.first((threadIdx.x >> 5) * gridDim.x + blockIdx.x);
+    p.next = p.seen = (uint32_t)min(base, (unsigned long long)R.limit);
+    p.end = p.next + 32u * R.per(0u);
+    p.dry = R.first(R.warps()) >= (unsigned long long)R.limit;
+    return p;
+}
+
+// The photon walk over medium M's range R, handed out by P, until it is used up. rk: the Philox round keys of M's seed (M.rk, or a copy
+// of them).
+template <int PHASE, bool SMEM_IMAGE, bool TRACE, class Range>
+__device__ __forceinline__ void walk_loop(const CommonArgs &C, const MediumArgs &M, const uint32_t (&rk)[20],
+                                          const Smem &S, const Range R, Pool P, Tally &T)
+{
     // camera transmittance exp(-mu_ext (ly/2 - r_y)) = 2^(cam_a r_y + cam_b)
     const float cam_a = M.mu_ext * 1.44269504088896340736f, cam_b = -cam_a * C.hy;
     uint32_t *s_img = S.img;
     unsigned long long *s_rad = S.rad, *s_tot = S.tot;
 
     // photon state
-    bool alive = false, done = false;
-    unsigned long long rel = 0;     // index within the medium's range
+    bool alive = false;
+    unsigned long long rel = 0;     // index within the medium's range (trace only)
     uint32_t pk0 = 0, pk1 = 0;      // global photon index, lo/hi words
     uint32_t ev = 0, ncoll = 0;
     float rx = 0, ry = 0, rz = 0, dx = 1, dy = 0, dz = 0, w = 1;
 
-    while (true) {
-        // -------- refill lanes whose photon ended
-        const unsigned need = __ballot_sync(FULL, !alive && !done);
-        if (need) {
-            const unsigned n_need = __popc(need);
-            const unsigned rank = __popc(need & lanemask_lt);
-            const unsigned long long avail = pool_end - pool_next;
-            unsigned long long mine;
-            if (avail >= n_need) {
-                mine = pool_next + rank;
-                pool_next += n_need;
-            } else {
-                unsigned long long base = 0;
-                if (lane == 0) base = grab();
-                base = __shfl_sync(FULL, base, 0);
-                mine = (rank < avail) ? pool_next + rank : base + (rank - avail);
-                pool_next = base + (n_need - avail);
-                pool_end = base + chunk;
-            }
-            if (!alive && !done) {
-                if (mine < limit) {
-                    rel = mine;
-                    const unsigned long long p = M.photon_offset + mine;
-                    pk0 = (uint32_t)p;
-                    pk1 = (uint32_t)(p >> 32);
-                    ev = 0;
-                    ncoll = 0;
-                    rx = 0.f; ry = 0.f; rz = 0.f;
-                    dx = 1.f; dy = 0.f; dz = 0.f;
-                    w = 1.f;
-                    if (C.beam_r > 0.f) {
-                        const uint4 b = philox10(make_uint4(pk0, pk1, 0xFFFFFFFFu, 0u), M.key0, M.key1);
-                        const float rho = C.beam_r * sqrtf(u01(b.x));
-                        float sp, cp;
-                        sincospif(2.0f * u01(b.y), &sp, &cp);
-                        ry = rho * cp;
-                        rz = rho * sp;
-                    }
-                    alive = true;
-                } else {
-                    done = true;
-                }
-            }
+    // a lane's next photon
+    auto start = [&](uint32_t mine) {
+        alive = true;
+        rel = mine;
+        const unsigned long long p = M.photon_offset + rel;
+        pk0 = (uint32_t)p;
+        pk1 = (uint32_t)(p >> 32);
+        ev = 0;
+        ncoll = 0;
+        rx = 0.f; ry = 0.f; rz = 0.f;
+        dx = 1.f; dy = 0.f; dz = 0.f;
+        w = 1.f;
+        if (C.beam_r > 0.f) {
+            const uint4 b = philox10(make_uint4(pk0, pk1, 0xFFFFFFFFu, 0u), M.key0, M.key1);
+            const float rho = C.beam_r * sqrtf(u01(b.x));
+            float sp, cp;
+            sincospif(2.0f * u01(b.y), &sp, &cp);
+            ry = rho * cp;
+            rz = rho * sp;
         }
-        if (!__any_sync(FULL, alive)) break;
+    };
+
+    while (true) {
+        const unsigned need = __ballot_sync(FULL, !alive);
+        if (need) {
+            const uint32_t mine = P.take(R, need);
+            if (!alive && mine < R.limit) start(mine);
+            if (!__any_sync(FULL, alive)) break;
+        }
         if (!alive) continue;
 
         // -------- one event
@@ -821,16 +896,11 @@ __global__ void __launch_bounds__(1024) walk_kernel(const __grid_constant__ Walk
         __syncthreads();
     }
     Tally T{0u, 0ll, 0ll, 0ll, 0ll, 0ll};
-    unsigned long long *counter = A.counter;
-    walk_loop<PHASE, SMEM_IMAGE, TRACE>(A.c, A.m, A.m.rk, S, A.m.n_photons, CHUNK,
-                                        [counter]() { return atomicAdd(counter, (unsigned long long)CHUNK); },
-                                        T);
+    const LaunchRange R{A.counter, (uint32_t)A.m.n_photons};
+    walk_loop<PHASE, SMEM_IMAGE, TRACE>(A.c, A.m, A.m.rk, S, R, launch_pool(R), T);
     flush<SMEM_IMAGE>(A.c, A.m, S, T);
 }
 
-// A batch counter holds the medium's next photon in its low bits and the
-// CTAs that joined the medium above them.
-constexpr unsigned long long JOIN = 1ull << 40;
 constexpr float JOIN_STEPS = 8192.f;   // photon-steps per CTA below which joining a running medium does not pay
 
 // The medium a CTA works on next (warp 0, all lanes): the one with most
@@ -879,7 +949,6 @@ __global__ void __launch_bounds__(1024) batch_kernel(const __grid_constant__ Bat
     __syncthreads();
     Tally T{0u, 0ll, 0ll, 0ll, 0ll, 0ll};
     uint32_t parity = 0;
-    const unsigned chunk = B.chunk;
     for (bool first = true;; first = false) {
         if (threadIdx.x < 32) {
             int m = -1;
@@ -893,12 +962,13 @@ __global__ void __launch_bounds__(1024) batch_kernel(const __grid_constant__ Bat
             }
             if (m < 0) m = pick_medium(B, threadIdx.x);
             if (threadIdx.x == 0) {
-                if (m >= 0) atomicAdd(B.counters + m, JOIN);
-                *S.item = (unsigned long long)(long long)m;
+                S.item[0] = (unsigned long long)(long long)m;
+                S.item[1] = m >= 0 ? atomicAdd(B.counters + m, JOIN) : 0ull;
             }
         }
         __syncthreads();
-        const int m = (int)(long long)*S.item;
+        const int m = (int)(long long)S.item[0];
+        const unsigned long long joined = S.item[1];
         __syncthreads();
         if (m < 0) break;
         // this medium's arguments, copied once: read through the dynamically
@@ -914,9 +984,12 @@ __global__ void __launch_bounds__(1024) batch_kernel(const __grid_constant__ Bat
         uint32_t rk[20];
 #pragma unroll
         for (int i = 0; i < 20; ++i) rk[i] = M.rk[i];
-        walk_loop<PHASE, SMEM_IMAGE, false>(
-            B.c, M, rk, S, M.n_photons, chunk,
-            [ctr, chunk]() { return atomicAdd(ctr, (unsigned long long)chunk) & (JOIN - 1); }, T);
+        const unsigned long long given = joined & (JOIN - 1);
+        const BatchRange R{ctr, (uint32_t)M.n_photons, B.max_per,
+                           0.5f / ((float)((uint32_t)(joined >> 40) + 1u) * (float)blockDim.x)};
+        Pool P;
+        P.seen = (uint32_t)min(given, (unsigned long long)R.limit);
+        walk_loop<PHASE, SMEM_IMAGE, false>(B.c, M, rk, S, R, P, T);
         flush<SMEM_IMAGE>(B.c, M, S, T);
         zero_tallies(S, B.c);
         __syncthreads();
@@ -1022,63 +1095,48 @@ __device__ __forceinline__ void grid_loop(const GridArgs &G, const Smem &S, cons
 {
     const CommonArgs &C = G.c;
     const MediumArgs &M = G.m;
-    const int lane = threadIdx.x & 31;
-    const unsigned lanemask_lt = (1u << lane) - 1u;
-    unsigned long long pool_next = 0, pool_end = 0;
+    const LaunchRange R{G.counter, (uint32_t)M.n_photons};
+    Pool P = launch_pool(R);
     uint32_t *s_img = S.img;
     unsigned long long *s_rad = S.rad, *s_tot = S.tot;
     const float INF = __int_as_float(0x7f800000);
 
-    bool alive = false, done = false;
+    bool alive = false;
     unsigned long long rel = 0;
     uint32_t pk0 = 0, pk1 = 0, ev = 0, ncoll = 0;
     float rx = 0, ry = 0, rz = 0, dx = 1, dy = 0, dz = 0, w = 1;
     float idx = 1, idy = INF, idz = INF;   // 1 / d (infinite along an axis d does not move on)
 
-    while (true) {
-        const unsigned need = __ballot_sync(FULL, !alive && !done);
-        if (need) {
-            const unsigned n_need = __popc(need), rank = __popc(need & lanemask_lt);
-            const unsigned long long avail = pool_end - pool_next;
-            unsigned long long mine;
-            if (avail >= n_need) {
-                mine = pool_next + rank;
-                pool_next += n_need;
-            } else {
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(G.counter, (unsigned long long)CHUNK);
-                base = __shfl_sync(FULL, base, 0);
-                mine = (rank < avail) ? pool_next + rank : base + (rank - avail);
-                pool_next = base + (n_need - avail);
-                pool_end = base + CHUNK;
-            }
-            if (!alive && !done) {
-                if (mine < M.n_photons) {
-                    rel = mine;
-                    const unsigned long long p = M.photon_offset + mine;
-                    pk0 = (uint32_t)p;
-                    pk1 = (uint32_t)(p >> 32);
-                    ev = 0;
-                    ncoll = 0;
-                    rx = 0.f; ry = 0.f; rz = 0.f;
-                    dx = 1.f; dy = 0.f; dz = 0.f;
-                    idx = 1.f; idy = INF; idz = INF;
-                    w = 1.f;
-                    if (C.beam_r > 0.f) {
-                        const uint4 b = philox10(make_uint4(pk0, pk1, 0xFFFFFFFFu, 0u), M.key0, M.key1);
-                        const float rho = C.beam_r * sqrtf(u01(b.x));
-                        float sp, cp;
-                        sincospif(2.0f * u01(b.y), &sp, &cp);
-                        ry = rho * cp;
-                        rz = rho * sp;
-                    }
-                    alive = true;
-                } else {
-                    done = true;
-                }
-            }
+    // a lane's next photon
+    auto start = [&](uint32_t mine) {
+        alive = true;
+        rel = mine;
+        const unsigned long long p = M.photon_offset + rel;
+        pk0 = (uint32_t)p;
+        pk1 = (uint32_t)(p >> 32);
+        ev = 0;
+        ncoll = 0;
+        rx = 0.f; ry = 0.f; rz = 0.f;
+        dx = 1.f; dy = 0.f; dz = 0.f;
+        idx = 1.f; idy = INF; idz = INF;
+        w = 1.f;
+        if (C.beam_r > 0.f) {
+            const uint4 b = philox10(make_uint4(pk0, pk1, 0xFFFFFFFFu, 0u), M.key0, M.key1);
+            const float rho = C.beam_r * sqrtf(u01(b.x));
+            float sp, cp;
+            sincospif(2.0f * u01(b.y), &sp, &cp);
+            ry = rho * cp;
+            rz = rho * sp;
         }
-        if (!__any_sync(FULL, alive)) break;
+    };
+
+    while (true) {
+        const unsigned need = __ballot_sync(FULL, !alive);
+        if (need) {
+            const uint32_t mine = P.take(R, need);
+            if (!alive && mine < R.limit) start(mine);
+            if (!__any_sync(FULL, alive)) break;
+        }
         if (!alive) continue;
 
         if (ev >= C.max_events) {
@@ -1409,7 +1467,6 @@ __global__ void __launch_bounds__(GADJ_BLOCK) grid_adjoint_kernel(const __grid_c
     }
 
     const int lane = threadIdx.x & 31;
-    const unsigned lanemask_lt = (1u << lane) - 1u;
     const float INF = __int_as_float(0x7f800000);
     // null scores: inside the box around the beam axis, this CTA's copy of
     // the voxel sums (many CTAs adding to the same voxels there at once
@@ -1422,8 +1479,9 @@ __global__ void __launch_bounds__(GADJ_BLOCK) grid_adjoint_kernel(const __grid_c
             return box + ((size_t)bz * A.bw + by) * G.gx + ix;
         return main + v;
     };
-    unsigned long long pool_next = 0, pool_end = 0;
-    bool alive = false, done = false;
+    const LaunchRange R{G.counter, (uint32_t)M.n_photons};
+    Pool pool = launch_pool(R);
+    bool alive = false;
     int pass = 0;
     uint32_t pk0 = 0, pk1 = 0, ev = 0, ncoll = 0;
     float rx = 0, ry = 0, rz = 0, dx = 1, dy = 0, dz = 0, w = 1;
@@ -1432,38 +1490,24 @@ __global__ void __launch_bounds__(GADJ_BLOCK) grid_adjoint_kernel(const __grid_c
     float P = 0.f, Ptot = 0.f;             // running / total camera terms of the photon
     double val = 0.0;
 
+    // a lane's next photon (its state is set at the start of a pass)
+    auto start = [&](uint32_t mine) {
+        alive = true;
+        const unsigned long long p = M.photon_offset + mine;
+        pk0 = (uint32_t)p;
+        pk1 = (uint32_t)(p >> 32);
+        pass = 0;
+        ev = 0;
+        ncoll = 0xFFFFFFFFu;
+    };
+
     while (true) {
-        const unsigned need = __ballot_sync(FULL, !alive && !done);
+        const unsigned need = __ballot_sync(FULL, !alive);
         if (need) {
-            const unsigned n_need = __popc(need), rank = __popc(need & lanemask_lt);
-            const unsigned long long avail = pool_end - pool_next;
-            unsigned long long mine;
-            if (avail >= n_need) {
-                mine = pool_next + rank;
-                pool_next += n_need;
-            } else {
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(G.counter, (unsigned long long)CHUNK);
-                base = __shfl_sync(FULL, base, 0);
-                mine = (rank < avail) ? pool_next + rank : base + (rank - avail);
-                pool_next = base + (n_need - avail);
-                pool_end = base + CHUNK;
-            }
-            if (!alive && !done) {
-                if (mine < M.n_photons) {
-                    const unsigned long long p = M.photon_offset + mine;
-                    pk0 = (uint32_t)p;
-                    pk1 = (uint32_t)(p >> 32);
-                    pass = 0;
-                    alive = true;
-                    ev = 0;   // the state itself is set below (start of a pass)
-                    ncoll = 0xFFFFFFFFu;
-                } else {
-                    done = true;
-                }
-            }
+            const uint32_t mine = pool.take(R, need);
+            if (!alive && mine < R.limit) start(mine);
+            if (!__any_sync(FULL, alive)) break;
         }
-        if (!__any_sync(FULL, alive)) break;
         int nseg = 0;          // stretches of the flight this lane queued this round
 
         if (alive && ncoll == 0xFFFFFFFFu) {
@@ -1771,11 +1815,10 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
     __syncthreads();
     const float c_s = A.c_s;   // 1/mu_s - 1/mu_ext
 
-    const unsigned lanemask_lt = (1u << lane) - 1u;
-    unsigned long long pool_next = 0, pool_end = 0;
-    bool alive = false, done = false;
+    const LaunchRange R{A.counter, (uint32_t)M.n_photons};
+    Pool pool = launch_pool(R);
+    bool alive = false;
     int pass = 1, cnt = 0;
-    unsigned long long rel = 0;
     uint32_t pk0 = 0, pk1 = 0, ev = 0, ncoll = 0;
     float rx = 0, ry = 0, rz = 0, dx = 1, dy = 0, dz = 0, w = 1, Ssc = 0;
     // the photon's running and total camera terms in single precision:
@@ -1792,37 +1835,22 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
 #pragma unroll
     for (int q = 0; q < ADJ_LIST; ++q) { lk[q] = 0; lf[q] = 0.0f; lp[q] = 0.0f; }
 
+    // a lane's next photon (its state is set at the start of a pass)
+    auto start = [&](uint32_t mine) {
+        alive = true;
+        const unsigned long long p = M.photon_offset + mine;
+        pk0 = (uint32_t)p;
+        pk1 = (uint32_t)(p >> 32);
+        pass = 1;
+    };
+
     while (true) {
-        const unsigned need = __ballot_sync(FULL, !alive && !done);
+        const unsigned need = __ballot_sync(FULL, !alive);
         if (need) {
-            const unsigned n_need = __popc(need), rank = __popc(need & lanemask_lt);
-            const unsigned long long avail = pool_end - pool_next;
-            unsigned long long mine;
-            if (avail >= n_need) {
-                mine = pool_next + rank;
-                pool_next += n_need;
-            } else {
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(A.counter, (unsigned long long)CHUNK);
-                base = __shfl_sync(FULL, base, 0);
-                mine = (rank < avail) ? pool_next + rank : base + (rank - avail);
-                pool_next = base + (n_need - avail);
-                pool_end = base + CHUNK;
-            }
-            if (!alive && !done) {
-                if (mine < M.n_photons) {
-                    rel = mine;
-                    const unsigned long long p = M.photon_offset + mine;
-                    pk0 = (uint32_t)p;
-                    pk1 = (uint32_t)(p >> 32);
-                    pass = 1;
-                    alive = true;
-                } else {
-                    done = true;
-                }
-            }
+            const uint32_t mine = pool.take(R, need);
+            if (!alive && mine < R.limit) start(mine);
+            if (!__any_sync(FULL, alive)) break;
         }
-        if (!__any_sync(FULL, alive)) break;
         if (!alive) continue;
         if (ev == 0) {
             // (re)start of a pass: the photon enters as in the forward walk
@@ -2042,7 +2070,7 @@ cudaError_t launch_sign_check(const WalkArgs &a, cudaStream_t st)
 }
 
 // Persistent grid: SMs x CTAs per SM (occupancy, or the caller's choice),
-// capped at what `work_warps` warps of work can use.
+// capped at what `work_warps` warps of work can use on all SMs.
 template <class Kern>
 cudaError_t launch_persistent(Kern kern, const void *args_unused, const LaunchCfg &cfg, size_t smem,
                               unsigned long long work_warps, unsigned *grid)
@@ -2060,14 +2088,17 @@ cudaError_t launch_persistent(Kern kern, const void *args_unused, const LaunchCf
     }
     unsigned long long blocks = (unsigned long long)sms * bps;
     const unsigned long long per_block = cfg.block / 32;
-    const unsigned long long cap = (work_warps + per_block - 1) / per_block;
+    unsigned long long cap = (work_warps + per_block - 1) / per_block;
+    const unsigned long long spread = work_warps < (unsigned long long)sms ? work_warps : (unsigned long long)sms;
+    if (cap < spread) cap = spread;   // few warps of work: over all SMs
     if (cap < blocks) blocks = cap;
     *grid = (unsigned)(blocks < 1 ? 1 : blocks);
     return cudaSuccess;
 }
 
-// Where the image accumulates and how big the CTA is. Sets c.band0/band_rows.
-cudaError_t plan_image(CommonArgs &c, LaunchCfg &cfg, bool *smem_img, size_t *smem)
+// Where the image accumulates and how big the CTA is for a launch over n_photons.
+// Sets c.band0/band_rows.
+cudaError_t plan_image(CommonArgs &c, LaunchCfg &cfg, unsigned long long n_photons, bool *smem_img, size_t *smem)
 {
     const size_t tb = ((c.phase_kind != MC_PHASE_HG) ? c.table_bytes : 0) + c.extra_bytes;
     const size_t tail = sizeof(unsigned long long) * (c.n_radial + MC_N_TOTALS + 3) + 16;
@@ -2108,7 +2139,15 @@ cudaError_t plan_image(CommonArgs &c, LaunchCfg &cfg, bool *smem_img, size_t *sm
         if (b0 > c.nz - c.band_rows) b0 = c.nz - c.band_rows;
         c.band0 = b0 < 0 ? 0 : b0;
     }
-    if (cfg.block == 0) cfg.block = (mode == 3) ? 1024 : 256;
+    // fewer photons than lanes on the chip: CTAs of as few warps (8 at least, for
+    // the tallies' clearing and flushing) as spread them over all SMs
+    if (cfg.block == 0) {
+        int sms = 0;
+        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        const unsigned long long warps = (n_photons + 31) / 32;
+        const unsigned long long per_sm_warps = (warps + sms - 1) / sms;
+        cfg.block = mode != 3 || per_sm_warps <= 8 ? 256 : (per_sm_warps >= 32 ? 1024 : 32 * (int)per_sm_warps);
+    }
     *smem = tb + tail + (*smem_img ? row * c.band_rows : 0);
     if (*smem > (size_t)optin) return cudaErrorInvalidValue;
     return cudaSuccess;
@@ -2119,7 +2158,7 @@ cudaError_t launch_one(const WalkArgs &a, const LaunchCfg &cfg, size_t smem, cud
 {
     auto kern = walk_kernel<PHASE, SMEM_IMAGE, TRACE>;
     unsigned grid = 0;
-    cudaError_t e = launch_persistent(kern, &a, cfg, smem, (a.m.n_photons + CHUNK - 1) / CHUNK, &grid);
+    cudaError_t e = launch_persistent(kern, &a, cfg, smem, (a.m.n_photons + 31) / 32, &grid);
     if (e != cudaSuccess) return e;
     kern<<<grid, cfg.block, smem, st>>>(a);
     return cudaGetLastError();
@@ -2130,8 +2169,8 @@ cudaError_t launch_batch_one(const BatchArgs &a, const LaunchCfg &cfg, size_t sm
 {
     auto kern = batch_kernel<PHASE, SMEM_IMAGE>;
     unsigned grid = 0;
-    unsigned long long chunks = 0;   // warp chunks of all media: more warps would idle
-    for (int i = 0; i < a.n_media; ++i) chunks += (a.m[i].n_photons + a.chunk - 1) / a.chunk;
+    unsigned long long chunks = 0;   // full warps of all media's photons: more would idle
+    for (int i = 0; i < a.n_media; ++i) chunks += (a.m[i].n_photons + 31) / 32;
     cudaError_t e = launch_persistent(kern, &a, cfg, smem, chunks, &grid);
     if (e != cudaSuccess) return e;
     kern<<<grid, cfg.block, smem, st>>>(a);
@@ -2144,7 +2183,7 @@ cudaError_t launch_grid_one(const GridArgs &a, const LaunchCfg &cfg, size_t smem
 {
     auto kern = grid_kernel<PHASE, SMEM_IMAGE, TRACE>;
     unsigned grid = 0;
-    cudaError_t e = launch_persistent(kern, &a, cfg, smem, (a.m.n_photons + CHUNK - 1) / CHUNK, &grid);
+    cudaError_t e = launch_persistent(kern, &a, cfg, smem, (a.m.n_photons + 31) / 32, &grid);
     if (e != cudaSuccess) return e;
     kern<<<grid, cfg.block, smem, st>>>(a);
     return cudaGetLastError();
@@ -2169,7 +2208,7 @@ cudaError_t launch_grid_adjoint_one(const GridAdjArgs &a, int rows, double *valu
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, GADJ_BLOCK, smem)) != cudaSuccess) return e;
     if (bps < 1) return cudaErrorInvalidConfiguration;
     long long grid = (long long)sms * bps;
-    const long long cap = (long long)((a.g.m.n_photons + CHUNK - 1) / CHUNK + GADJ_BLOCK / 32 - 1) / (GADJ_BLOCK / 32);
+    const long long cap = (long long)((a.g.m.n_photons + 31) / 32 + GADJ_BLOCK / 32 - 1) / (GADJ_BLOCK / 32);
     if (cap < grid) grid = cap < 1 ? 1 : cap;
     if (grid > rows) grid = rows;
     kern<<<(unsigned)grid, GADJ_BLOCK, smem, st>>>(a);
@@ -2215,7 +2254,7 @@ cudaError_t launch_walk(const WalkArgs &a0, bool trace, const LaunchCfg &cfg0, c
     LaunchCfg cfg = cfg0;
     bool smem_img = false;
     size_t smem = 0;
-    cudaError_t e = plan_image(a.c, cfg, &smem_img, &smem);
+    cudaError_t e = plan_image(a.c, cfg, a.m.n_photons, &smem_img, &smem);
     if (e != cudaSuccess) return e;
     if ((e = launch_walk_kernel(a, trace, cfg, smem_img, smem, st)) != cudaSuccess) return e;
     return launch_sign_check(a, st);
@@ -2227,7 +2266,7 @@ cudaError_t check_plan(const CommonArgs &c0, const LaunchCfg &cfg0)
     LaunchCfg cfg = cfg0;
     bool smem_img = false;
     size_t smem = 0;
-    return plan_image(c, cfg, &smem_img, &smem);
+    return plan_image(c, cfg, 0, &smem_img, &smem);
 }
 
 namespace {
@@ -2258,7 +2297,7 @@ cudaError_t launch_grid(const GridArgs &a0, bool trace, const LaunchCfg &cfg0, c
     LaunchCfg cfg = cfg0;
     bool smem_img = false;
     size_t smem = 0;
-    cudaError_t e = plan_image(a.c, cfg, &smem_img, &smem);
+    cudaError_t e = plan_image(a.c, cfg, a.m.n_photons, &smem_img, &smem);
     if (e != cudaSuccess) return e;
     if ((e = launch_grid_kernel(a, trace, cfg, smem_img, smem, st)) != cudaSuccess) return e;
     WalkArgs w;
@@ -2306,12 +2345,12 @@ cudaError_t launch_batch(const BatchArgs &a0, bool fresh, const LaunchCfg &cfg0,
     LaunchCfg cfg = cfg0;
     bool smem_img = false;
     size_t smem = 0;
-    cudaError_t e = plan_image(a.c, cfg, &smem_img, &smem);
+    unsigned long long photons = 0;
+    for (int i = 0; i < a.n_media; ++i) photons += a.m[i].n_photons;
+    cudaError_t e = plan_image(a.c, cfg, photons, &smem_img, &smem);
     if (e != cudaSuccess) return e;
-    bool any = false;
-    for (int i = 0; i < a.n_media; ++i) any |= a.m[i].n_photons != 0;
     batch_zero_kernel<<<dim3(fresh ? sign_blocks(a.c) : 1, (unsigned)a.n_media), ZERO_BLOCK, 0, st>>>(a, fresh);
-    if ((e = cudaGetLastError()) != cudaSuccess || !any) return e;
+    if ((e = cudaGetLastError()) != cudaSuccess || !photons) return e;
     switch (a.c.phase_kind * 2 + (smem_img ? 1 : 0)) {
     case 0: e = launch_batch_one<MC_PHASE_TABLE, false>(a, cfg, smem, st); break;
     case 1: e = launch_batch_one<MC_PHASE_TABLE, true>(a, cfg, smem, st); break;
@@ -2352,7 +2391,7 @@ cudaError_t launch_adjoint_one(const AdjArgs &a, int rows, double *out, cudaStre
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, block, smem)) != cudaSuccess) return e;
     if (bps < 1) return cudaErrorInvalidConfiguration;
     long long grid = (long long)sms * bps;
-    const long long cap = (long long)((a.m.n_photons + CHUNK - 1) / CHUNK + block / 32 - 1) / (block / 32);
+    const long long cap = (long long)((a.m.n_photons + 31) / 32 + block / 32 - 1) / (block / 32);
     if (cap < grid) grid = cap < 1 ? 1 : cap;
     if (grid > rows) grid = rows;
     if (PHASEW) {
