@@ -171,7 +171,8 @@ void fill_common(mcx::CommonArgs &c, const mc_medium *m, const mc_geometry *g, c
     c.rr_surv = (float)r->rr_survival;
     c.inv_rr_surv = r->rr_survival > 0 ? (float)(1.0 / r->rr_survival) : 0.0f;
     c.max_events = r->max_events;
-    c.max_scatter = r->max_scatter;
+    c.scatter_cap = r->max_scatter ? r->max_scatter : 0xFFFFFFFFu;
+    c.ev_stop = std::min(c.max_events, c.scatter_cap);
     c.img_scale = std::ldexp(1.0f, frac_bits_of(r, n_photons));
     c.error = error;
     c.extra_bytes = 0;

@@ -41,12 +41,15 @@ struct CommonArgs {
     float sx, sz, sr;           // nx/lx, nz/lz, n_radial/r_max
     // run
     float rr_thr, rr_surv, inv_rr_surv;
-    uint32_t max_events, max_scatter;
+    uint32_t max_events;
+    uint32_t scatter_cap;       // collisions a photon may have (max_scatter, or 2^32 - 1 for none)
+    uint32_t ev_stop;           // min(max_events, scatter_cap)
     float img_scale;            // 2^image_frac_bits
     uint32_t *error;
     // image rows [band0, band0 + band_rows) are privatised in shared memory
     // (set by the launcher; band_rows = nz for a whole-image tile)
     int band0, band_rows;
+    int band_first, band_pixels;   // the same as pixels
     // trace (trace kernels only)
     int32_t *trace;
     int n_trace, n_trace_events;
