@@ -17,7 +17,7 @@
 // What bounds them: GB300 issues 2 double-precision instructions per clock
 // and SM, and one CTA per image or ring (the earlier layout: a division per
 // pixel in each of n_r + 2 passes) left most SMs idle: a call on three
-// 512 x 512 images with 32 rings took 4.87 ms, now 0.157 ms (the read-back
+// 512 x 512 images with 32 rings took 4.87 ms, now 0.110 ms (the read-back
 // of the numbers included). The scan uses no double-precision arithmetic but
 // for pixels next to a ring's edge, the pair pass about 24 such instructions
 // per pixel.
@@ -37,7 +37,7 @@ constexpr int RUN = 8;         // consecutive pixels per scan thread: a ring is 
 constexpr int MAX_RINGS = 4096;
 constexpr int SMEM_RINGS = 512;   // rings summed in shared memory first (26 KB); beyond, ring sums are spread
                                   // over so many addresses that L2 takes them directly
-constexpr int MAX_PAIR_CTAS = 592;
+constexpr int MAX_PAIR_CTAS = 304;   // two per SM: a CTA's start and end cost about as much as 6 pixels a thread
 constexpr unsigned FULL = 0xffffffffu;
 
 struct Imgs {
@@ -218,26 +218,32 @@ __device__ __forceinline__ double norm_sum(u64 lo, u64 hi, long long cnt, const 
     return fma((double)top, 4294967296.0, (double)low) / n.range;
 }
 
-// v[0..K) summed over the CTA in a fixed order (lanes, then warps); every
-// thread gets the sums. red: MB / 32 * K doubles.
+// v[0..K) of the first `warps` warps summed in a fixed order (lanes, then
+// warps); every thread gets the sums. One lane per value adds the warps' sums:
+// each double-precision instruction holds an SM's pipe for 16 clocks a warp.
+// red: (MB / 32 + 1) * K doubles.
 template <int K>
-__device__ __forceinline__ void block_sums(double (&v)[K], double *red)
+__device__ __forceinline__ void block_sums(double (&v)[K], double *red, int warps = MB / 32)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(FULL, v[k], o);
     __syncthreads();
-    if (lane == 0)
+    if (warp < warps) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) red[warp * K + k] = v[k];
-    __syncthreads();
+        for (int k = 0; k < K; ++k)
+            for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(FULL, v[k], o);
+        if (lane == 0)
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        double t = 0.0;
-        for (int q = 0; q < MB / 32; ++q) t += red[q * K + k];
-        v[k] = t;
+            for (int k = 0; k < K; ++k) red[K + warp * K + k] = v[k];
     }
+    __syncthreads();
+    if (threadIdx.x < K) {
+        double t = 0.0;
+        for (int q = 0; q < warps; ++q) t += red[K + q * K + threadIdx.x];
+        red[threadIdx.x] = t;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; ++k) v[k] = red[k];
 }
 
 // Images 1 .. NI-1 against image 0 (the reference); partials: [CTA][7] rows of
@@ -247,14 +253,22 @@ template <int NI>
 __global__ void __launch_bounds__(MB) pair_kernel(Imgs im, long long npix, int n_r, Scan *sc, Rings R,
                                                   double *partials, double *out)
 {
-    __shared__ double red[MB / 32 * 16];
+    __shared__ double red[(MB / 32 + 1) * 16];
     __shared__ bool last;
+    __shared__ Norm s_nm[NI];
+    __shared__ double s_mean[NI];
+    if (threadIdx.x < NI) {     // one lane per image: three divisions each
+        const int k = threadIdx.x;
+        s_nm[k] = norm_of(sc, k);
+        s_mean[k] = norm_sum(sc->tot_lo[k], sc->tot_hi[k], npix, s_nm[k]) / (double)npix;
+    }
+    __syncthreads();
     Norm nm[NI];
     double mean[NI];
 #pragma unroll
     for (int k = 0; k < NI; ++k) {
-        nm[k] = norm_of(sc, k);
-        mean[k] = norm_sum(sc->tot_lo[k], sc->tot_hi[k], npix, nm[k]) / (double)npix;
+        nm[k] = s_nm[k];
+        mean[k] = s_mean[k];
     }
     double acc[7];
 #pragma unroll
@@ -285,7 +299,8 @@ __global__ void __launch_bounds__(MB) pair_kernel(Imgs im, long long npix, int n
     for (int q = 0; q < 7; ++q) acc[q] = 0.0;
     for (int r = threadIdx.x; r < (int)gridDim.x; r += MB)
         for (int q = 0; q < 7; ++q) acc[q] += __ldcg(&partials[(size_t)r * 7 + q]);
-    block_sums(acc, red);
+    const int row_warps = min((int)(gridDim.x + 31) / 32, MB / 32), ring_warps = min((n_r + 31) / 32, MB / 32);
+    block_sums(acc, red, row_warps);
     double *prof = out + 13;   // [3][n_r]
     // sums over the rings that hold pixels: their number, profiles, the
     // profiles' squared differences and ring counts by zone, rings where
@@ -317,7 +332,7 @@ __global__ void __launch_bounds__(MB) pair_kernel(Imgs im, long long npix, int n
         else v[12] += 1.0;
         if (NI == 3 && fabs(p[1] - p[0]) < fabs(p[2] - p[0])) v[13] += 1.0;
     }
-    block_sums(v, red);
+    block_sums(v, red, ring_warps);
     double c[5] = {0.0, 0.0, 0.0, 0.0, 0.0};   // centred profile products: reference, then cross and auto per pair
     for (int b = threadIdx.x; b < n_r; b += MB) {
         if (!R.cnt[b]) continue;
@@ -330,7 +345,7 @@ __global__ void __launch_bounds__(MB) pair_kernel(Imgs im, long long npix, int n
             c[2 * k] += da * da;
         }
     }
-    block_sums(c, red);
+    block_sums(c, red, ring_warps);
     if (threadIdx.x < 2) {   // one thread per pair
         const int p = threadIdx.x;
         double *o = out + 6 * p;
