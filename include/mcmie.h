@@ -417,7 +417,8 @@ mc_status mc_run_grid(const mc_grid *grid, const void *d_grid_work, const mc_med
  * depend on scheduling); *d_value = L
  * (double, fixed order).
  * d_work: mc_grid_adjoint_workspace_bytes(grid) bytes (three
- * double-precision voxel arrays). The kernel holds the phase table, the
+ * double-precision voxel arrays, and copies of the part of them around the
+ * beam axis). The kernel holds the phase table, the
  * majorant cells and 12 KB of per-warp flight queues in shared memory: a
  * table and cell count that do not fit there (the largest table with the
  * most cells does not) are refused with MC_ERR_ARG before anything runs.

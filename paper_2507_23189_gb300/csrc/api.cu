@@ -676,6 +676,14 @@ mc_status mc_run_grid(const mc_grid *g, const void *d_grid_work, const mc_medium
     return cuda_status(mcx::launch_grid(a, d_trace != nullptr, launch_cfg(run), st));
 }
 
+// Voxels in the gradients' box around the beam axis: all x, the central
+// min(kBoxWidth, gy, gz) voxels along y and z.
+static size_t box_voxels(const mc_grid *g)
+{
+    const size_t bw = (size_t)std::min(mcx::kBoxWidth, std::min(g->gy, g->gz));
+    return (size_t)g->gx * bw * bw;
+}
+
 size_t mc_grid_adjoint_workspace_bytes(const mc_grid *g)
 {
     int mx, my, mz;
@@ -683,16 +691,11 @@ size_t mc_grid_adjoint_workspace_bytes(const mc_grid *g)
     const int rows = mcx::grid_adjoint_max_grid();
     if (rows < 1) return 0;
     const size_t n = (size_t)g->gx * g->gy * g->gz;
-    // voxel sum, column sources, first-flight row entries
-    return kAlign + 3 * up(sizeof(double) * n) + up(sizeof(double) * (size_t)rows);
-}
-
-// Voxels in the null-score gradient's box around the beam axis: all x, the
-// central min(kNullBox, gy, gz) voxels along y and z.
-static size_t null_box(const mc_grid *g)
-{
-    const size_t bw = (size_t)std::min(mcx::kNullBox, std::min(g->gy, g->gz));
-    return (size_t)g->gx * bw * bw;
+    // voxel sum, column sources, first-flight row entries; kBoxCopies copies of
+    // the first two over the box around the beam axis, kRowCopies of the beam's
+    // row of the third
+    return kAlign + 3 * up(sizeof(double) * n) + 2 * (size_t)mcx::kBoxCopies * up(sizeof(double) * box_voxels(g)) +
+           up(sizeof(double) * (size_t)mcx::kRowCopies * g->gx) + up(sizeof(double) * (size_t)rows);
 }
 
 size_t mc_grid_adjoint_nulls_workspace_bytes(const mc_grid *g)
@@ -702,9 +705,9 @@ size_t mc_grid_adjoint_nulls_workspace_bytes(const mc_grid *g)
     const int rows = mcx::grid_adjoint_max_grid();
     if (rows < 1) return 0;
     const size_t n = (size_t)g->gx * g->gy * g->gz;
-    // the voxel sum and the column sources, and kNullCopies copies of each
+    // the voxel sum and the column sources, and kBoxCopies copies of each
     // over the box around the beam axis
-    return kAlign + 2 * up(sizeof(double) * n) + 2 * (size_t)mcx::kNullCopies * up(sizeof(double) * null_box(g)) +
+    return kAlign + 2 * up(sizeof(double) * n) + 2 * (size_t)mcx::kBoxCopies * up(sizeof(double) * box_voxels(g)) +
            up(sizeof(double) * (size_t)rows);
 }
 
@@ -759,24 +762,27 @@ mc_status grid_adjoint_common(const mc_grid *g, const void *d_grid_work, const m
     std::memset(&a, 0, sizeof a);
     fill_grid(a.g, g, mx, my, mz, d_grid_work, &m, geom, camera, run, d_error, nullptr, nullptr, nullptr);
     const size_t nb = up(sizeof(double) * n);
-    // exact: s1, ex, gsum; null scores: s1, gsum, then the box copies of s1
-    // and of gsum
-    const int bw = std::min(mcx::kNullBox, std::min(g->gy, g->gz));
-    const size_t bb = up(sizeof(double) * null_box(g));
-    const size_t region = nulls ? 2 * nb + 2 * (size_t)mcx::kNullCopies * bb : 3 * nb;
+    // s1, gsum (exact: and ex), the box copies of s1 and of gsum (exact: and
+    // the row copies of ex)
+    const int bw = std::min(mcx::kBoxWidth, std::min(g->gy, g->gz));
+    const size_t bb = up(sizeof(double) * box_voxels(g)), cb = (size_t)mcx::kBoxCopies * bb;
+    const size_t rb = up(sizeof(double) * (size_t)mcx::kRowCopies * g->gx);
+    const size_t main = (nulls ? 2 : 3) * nb, region = main + 2 * cb + (nulls ? 0 : rb);
+    auto at = [&](size_t off) { return reinterpret_cast<double *>(w + kAlign + off); };
     a.g.counter = reinterpret_cast<unsigned long long *>(w);
-    a.s1 = reinterpret_cast<double *>(w + kAlign);
-    a.ex = nulls ? nullptr : reinterpret_cast<double *>(w + kAlign + nb);
-    a.gsum = reinterpret_cast<double *>(w + kAlign + (nulls ? 1 : 2) * nb);
-    a.bs1 = nulls ? reinterpret_cast<double *>(w + kAlign + 2 * nb) : nullptr;
-    a.bgs = nulls ? reinterpret_cast<double *>(w + kAlign + 2 * nb + mcx::kNullCopies * bb) : nullptr;
-    a.copies = nulls ? mcx::kNullCopies : 1;
-    a.bw = nulls ? bw : 0;
+    a.s1 = at(0);
+    a.gsum = at(nb);
+    a.ex = nulls ? nullptr : at(2 * nb);
+    a.bs1 = at(main);
+    a.bgs = at(main + cb);
+    a.exr = nulls ? nullptr : at(main + 2 * cb);
+    a.copies = mcx::kBoxCopies;
+    a.bw = bw;
     a.by0 = g->gy / 2 - bw / 2;   // centred on the beam axis (y = z = 0)
     a.bz0 = g->gz / 2 - bw / 2;
-    a.nbox = null_box(g);
+    a.nbox = box_voxels(g);
     a.bstride = bb / sizeof(double);
-    a.partials = reinterpret_cast<double *>(w + kAlign + region);
+    a.partials = at(region);
     a.adj = d_adj_image;
     a.grad = d_grad;
     a.k_ext = (float)g->k_ext;

@@ -119,11 +119,12 @@ struct GridAdjArgs {
     const float *adj;             // [nz][nx]
     // [gz][gy][gx] double-precision atomic sums: point, flight and own-voxel
     // column terms; column sources above a collision; first-flight row suffix.
-    // With null scores, the voxels of the box iy in [by0, by0 + bw), iz in
-    // [bz0, bz0 + bw) around the beam axis (where many CTAs add at once) are
-    // summed instead in `copies` copies of the box, bstride elements apart,
-    // CTA b adding into copy b % copies: bgs for gsum, bs1 for s1
-    double *gsum, *s1, *ex;
+    // The voxels of the box iy in [by0, by0 + bw), iz in [bz0, bz0 + bw)
+    // around the beam axis (where many CTAs add at once) are summed in
+    // `copies` copies of the box, bstride elements apart, CTA b adding into
+    // copy b % copies: bgs for gsum, bs1 for s1; the row suffix of the beam's
+    // own row in kRowCopies rows exr
+    double *gsum, *s1, *ex, *exr;
     double *bgs, *bs1;
     int copies, by0, bz0, bw;
     size_t nbox, bstride;
@@ -176,9 +177,10 @@ cudaError_t grid_adjoint_check(const GridAdjArgs &a);
 
 // grad[v] = gsum[v] + vx * (sum of ex after v in its row along x)
 //           - k_ext vy * (sum of s1 below v in its column along y); gsum is
-// updated in place by the row sums; ex null: no row terms.
-cudaError_t launch_gradient_fold(double *gsum, const double *s1, const double *ex, float *grad, int gx, int gy,
-                                 int gz, double k_ext, double vx, double vy, cudaStream_t stream);
+// updated in place by the row sums; ex null: no row terms. exr: kRowCopies
+// further rows of ex for the row (gy / 2, gz / 2).
+cudaError_t launch_gradient_fold(double *gsum, const double *s1, const double *ex, const double *exr, float *grad,
+                                 int gx, int gy, int gz, double k_ext, double vx, double vy, cudaStream_t stream);
 
 // gsum[v] += sum over the copies of bgs at v's box element, s1 likewise
 // (copies bstride elements apart, summed in copy order).
@@ -186,10 +188,12 @@ cudaError_t launch_box_merge(double *gsum, double *s1, const double *bgs, const 
                              size_t nbox, size_t bstride, int gx, int gy, int by0, int bz0, int bw,
                              cudaStream_t stream);
 
-// The null-score gradient's copies of the voxel sums near the beam axis: how
-// many, and the box's width in voxels along y and z (at most the grid's).
-constexpr int kNullCopies = 8;
-constexpr int kNullBox = 32;
+// The gradients' copies of the voxel sums near the beam axis: how many, the
+// box's width in voxels along y and z (at most the grid's), and the copies of
+// the beam's row of first flights.
+constexpr int kBoxCopies = 8;
+constexpr int kBoxWidth = 32;
+constexpr int kRowCopies = 32;
 
 // CTAs the grid adjoint may use on the current device (for workspace sizing).
 int grid_adjoint_max_grid();

@@ -65,8 +65,9 @@ __global__ void __launch_bounds__(256) majorant_kernel(const float *__restrict__
 // one where a first flight ended takes the full voxel length vx of that
 // flight's coefficient, gsum[ix] += vx * sum_{j > ix} ex[j]. Chunks of 32
 // voxels with a warp suffix scan; rows with no entries cost their loads.
-__global__ void row_suffix_kernel(double *__restrict__ gsum, const double *__restrict__ ex, int gx,
-                                  long long rows, double vx)
+__global__ void row_suffix_kernel(double *__restrict__ gsum, const double *__restrict__ ex,
+                                  const double *__restrict__ exr, long long beam_row, int gx, long long rows,
+                                  double vx)
 {
     const long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
     if (r >= rows) return;   // whole warps leave together
@@ -75,7 +76,10 @@ __global__ void row_suffix_kernel(double *__restrict__ gsum, const double *__res
     double carry = 0.0;      // sum of ex beyond the current chunk
     for (int c = ((gx - 1) >> 5) << 5; c >= 0; c -= 32) {
         const int ix = c + lane;
-        const double e = ix < gx ? ex[base + ix] : 0.0;
+        double e = ix < gx ? ex[base + ix] : 0.0;
+        if (r == beam_row && ix < gx)
+#pragma unroll 8
+            for (int k = 0; k < kRowCopies; ++k) e += exr[(size_t)k * gx + ix];
         if (__any_sync(0xFFFFFFFFu, e != 0.0)) {
             double s = e;    // inclusive suffix within the chunk
             for (int o = 1; o < 32; o <<= 1) {
@@ -142,13 +146,14 @@ cudaError_t launch_box_merge(double *gsum, double *s1, const double *bgs, const 
     return cudaGetLastError();
 }
 
-cudaError_t launch_gradient_fold(double *gsum, const double *s1, const double *ex, float *grad, int gx, int gy,
-                                 int gz, double k_ext, double vx, double vy, cudaStream_t st)
+cudaError_t launch_gradient_fold(double *gsum, const double *s1, const double *ex, const double *exr, float *grad,
+                                 int gx, int gy, int gz, double k_ext, double vx, double vy, cudaStream_t st)
 {
     cudaError_t e;
     if (ex) {
         const long long rows = (long long)gy * gz;
-        row_suffix_kernel<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, st>>>(gsum, ex, gx, rows, vx);
+        row_suffix_kernel<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, st>>>(
+            gsum, ex, exr, (long long)(gz / 2) * gy + gy / 2, gx, rows, vx);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     const long long cols = (long long)gx * gz;

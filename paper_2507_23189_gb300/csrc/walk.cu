@@ -1327,23 +1327,20 @@ __global__ void __launch_bounds__(1024) grid_kernel(const __grid_constant__ Grid
 // double-precision pipe, a small fraction of the single-precision rate,
 // is not used on this path.
 constexpr int GADJ_BLOCK = 256;
-// per-warp queue of flights to rasterise, one column per lane: for the three
-// axes in partition order, the first crossing distance and the spacing of
-// the plane crossings, and the count with the axis code; then the length,
-// the coefficient and the start voxel
+// per-warp queue of flights to rasterise, one column per lane: for x, y and z
+// the first crossing distance, the spacing of the plane crossings and the count
+// with the direction; then the length, the coefficient and the start voxel
 constexpr int GADJ_SEG = 12;
 
-// float -> double by moving the bit fields: exact for normal numbers and
-// infinities; subnormals (far below any term summed here) become zero.
+// float -> double by moving the bit fields, on the integer pipe (GB300's
+// double-precision pipe, which converts, takes 2 lanes per clock and SM):
+// exact for normal numbers, infinities and NaN; zero and subnormals come out
+// below 2^-126, far under any term summed here.
 __device__ __forceinline__ double widen(float f)
 {
-    const uint32_t u = __float_as_uint(f);
-    const uint32_t e = (u >> 23) & 0xFFu;
-    const uint32_t s = u & 0x80000000u;
-    const uint32_t ex = e == 0xFFu ? 0x7FFu : e + 896u;     // rebias 127 -> 1023
-    const uint32_t hi = e == 0u ? s : (s | (ex << 20) | ((u & 0x7FFFFFu) >> 3));
-    const uint32_t lo = e == 0u ? 0u : (u << 29);
-    return __hiloint2double((int)hi, (int)lo);
+    const int hi = (int)(((uint32_t)(__float_as_int(f) >> 3) & 0x8FFFFFFFu) + 0x38000000u);   // exponent + 896
+    const int lo = (int)(__float_as_uint(f) << 29);
+    return __hiloint2double(fabsf(f) < __int_as_float(0x7f800000) ? hi : hi | 0x7FF00000, lo);
 }
 
 __device__ __forceinline__ float rcp_approx(float x)
@@ -1371,83 +1368,84 @@ struct Cross {
     bool up;
 };
 
+// The crossings among 0 .. n-1 at distances < t (LE: <= t), idl about 1 / dl.
+// The product is off by less than one crossing (2^-21 of at most 4096), so one
+// step mends it.
+template <bool LE>
+__device__ __forceinline__ int count_to(float t0, float dl, float idl, int n, float t)
+{
+    int c = min(max(__float2int_rd((t - t0) * idl) + 1, 0), n);
+    const float below = cross_at(t0, dl, c - 1), above = cross_at(t0, dl, c);
+    if (c > 0 && !(LE ? below <= t : below < t)) --c;
+    else if (c < n && (LE ? above <= t : above < t)) ++c;
+    return c;
+}
+
 __device__ __forceinline__ Cross axis_cross(float p, float d, float id, float lo, float v, float iv, int g,
                                             float len)
 {
     Cross c;
     c.i0 = min(max(__float2int_rd((p - lo) * iv), 0), g - 1);
     c.up = d > 0.f;
-    c.t0 = 0.f;
+    c.t0 = __int_as_float(0x7f800000);
     c.dl = 1.f;
     c.n = 0;
-    if (!(fabsf(id) < __int_as_float(0x7f800000))) return c;   // no motion along this axis
+    if (!(fabsf(id) < __int_as_float(0x7f800000))) return c;   // no motion along this axis: no crossing
     c.t0 = (fmaf((float)(c.up ? c.i0 + 1 : c.i0), v, lo) - p) * id;
     c.dl = v * fabsf(id);
-    const int lim = c.up ? g - 1 - c.i0 : c.i0;
-    int n = min(max(__float2int_ru((len - c.t0) * (fabsf(d) * iv)), 0), lim);
-    while (n > 0 && !(cross_at(c.t0, c.dl, n - 1) < len)) --n;
-    while (n < lim && cross_at(c.t0, c.dl, n) < len) ++n;
-    c.n = n;
+    c.n = count_to<false>(c.t0, c.dl, fabsf(d) * iv, c.up ? g - 1 - c.i0 : c.i0, len);
     return c;
 }
 
-// crossings of an axis at distances <= t, and the distance of the next one
-__device__ __forceinline__ int count_le(float t0, float dl, int n, float t, float &next)
+// Unit u of the `units` that queued flight q is cut into, equal lengths of it:
+// the pieces between consecutive plane crossings (of any axis) that end in the
+// unit's stretch (the flight's own end closes the last); grad[voxel] += coef *
+// length of each. Crossings are evenly spaced on every axis, so the units of a
+// flight hold the same number of pieces within a few, and a piece belongs to
+// one unit whole. Axes crossed at the same distance advance together. No
+// crossing past an axis's count lies before the flight's end (see the queue).
+__device__ __forceinline__ void raster_unit(const GridAdjArgs &A, double *bgs, const float *s_seg, int q, int u,
+                                            int units)
 {
-    int c = 0;
-    if (n > 0) {
-        c = min(max(__float2int_rd((t - t0) * rcp_approx(dl)) + 1, 0), n);
-        while (c > 0 && cross_at(t0, dl, c - 1) > t) --c;
-        while (c < n && cross_at(t0, dl, c) <= t) ++c;
-    }
-    next = c < n ? cross_at(t0, dl, c) : __int_as_float(0x7f800000);
-    return c;
-}
-
-// Unit u of queued flight q: the stretch between crossings u-1 and u of its
-// partition axis A (the axis it crosses most; the flight's start and end
-// close the first and last stretch), walked across the crossings of the
-// other two axes B and C inside it; grad[voxel] += coef * length of each
-// piece.
-__device__ __forceinline__ void raster_unit(const GridArgs &G, double *grad, const float *s_seg, int q, int u)
-{
-    const float INF = __int_as_float(0x7f800000);
+    const GridArgs &G = A.g;
     const float *f = s_seg + q;
     const int *fi = reinterpret_cast<const int *>(f);
-    const int wA = fi[192], wB = fi[224], wC = fi[256];
-    const int nA = wA & 0xFFFF, nB = wB & 0xFFFF, nC = wC & 0xFFFF;
-    auto stride = [&](int w) {
-        const int ax = (w >> 16) & 3;
-        const int st = ax == 0 ? 1 : (ax == 1 ? G.gx : G.gx * G.gy);
-        return (w >> 18) & 1 ? -st : st;
-    };
-    const float len = f[288], coef = f[320];
-    const float tB0 = f[32], dB = f[128], tC0 = f[64], dC = f[160];
-    const float t0 = u == 0 ? 0.f : cross_at(f[0], f[96], u - 1);
-    const float t1 = u == nA ? len : cross_at(f[0], f[96], u);
-    float nextB, nextC;
-    int cB = count_le(tB0, dB, nB, t0, nextB);
-    int cC = count_le(tC0, dC, nC, t0, nextC);
-    const int sB = stride(wB), sC = stride(wC);
-    int v = fi[352] + u * stride(wA) + cB * sB + cC * sC;
-    float t = t0;
-    for (int it = 0; it <= nB + nC; ++it) {
-        const bool bfirst = nextB <= nextC;
-        const float m = fminf(nextB, nextC);
-        const float e = fminf(m, t1);
-        if (e > t) atomicAdd(&grad[chk(v, G.gx * G.gy * G.gz, G.c.error)], widen(coef * (e - t)));
-        t = e;
-        if (!(m < t1)) break;
-        if (bfirst) {
-            v += sB;
-            ++cB;
-            nextB = cB < nB ? cross_at(tB0, dB, cB) : INF;
-        } else {
-            v += sC;
-            ++cC;
-            nextC = cC < nC ? cross_at(tC0, dC, cC) : INF;
-        }
+    const float coef = f[320];
+    const bool last = u == units - 1, box = fi[64] >> 17;
+    double *grad = box ? bgs : A.gsum;
+    const int span = box ? (int)A.nbox : G.gx * G.gy * G.gz;
+    const float step = f[288] * rcp_approx((float)units);
+    const float t0 = (float)u * step, t1 = last ? f[288] : (float)(u + 1) * step;
+    int v = fi[352];
+    float t = 0.f, next[3], dl[3], first[3], j[3];
+    int st[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        first[a] = f[96 * a];
+        dl[a] = f[96 * a + 32];
+        const int w = fi[96 * a + 64];
+        st[a] = a == 0 ? 1 : (a == 1 ? G.gx : G.gx * (box ? A.bw : G.gy));
+        if ((w >> 16) & 1) st[a] = -st[a];
+        const int c = u ? count_to<true>(first[a], dl[a], rcp_approx(dl[a]), w & 0xFFFF, t0) : 0;
+        if (c > 0) t = fmaxf(t, cross_at(first[a], dl[a], c - 1));
+        v += c * st[a];
+        j[a] = (float)c;   // below 4096: the next distance is one FMA
+        next[a] = cross_at(first[a], dl[a], c);
     }
+    for (int it = 0; it < 3 * 4096; ++it) {
+        const float m = fminf(fminf(next[0], next[1]), next[2]);
+        if (!(m <= t1)) break;
+        if (m > t) atomicAdd(&grad[chk(v, span, G.c.error)], widen(coef * (m - t)));
+        t = m;
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            if (next[a] == m) {
+                v += st[a];
+                j[a] += 1.f;
+                next[a] = fmaxf(fmaf(j[a], dl[a], first[a]), 0.f);
+            }
+    }
+    if (last && t1 > t) atomicAdd(&grad[chk(v, span, G.c.error)], widen(coef * (t1 - t)));
 }
 
 // NULLS: the flights' transmission is scored at the null collisions of
@@ -1459,7 +1457,7 @@ __device__ __forceinline__ void raster_unit(const GridArgs &G, double *grad, con
 // collision replaces the rasterised flight; both are unbiased estimates of
 // the same gradient.
 template <int PHASE, bool NULLS>
-__global__ void __launch_bounds__(GADJ_BLOCK) grid_adjoint_kernel(const __grid_constant__ GridAdjArgs A)
+__global__ void __launch_bounds__(GADJ_BLOCK, NULLS ? 0 : 4) grid_adjoint_kernel(const __grid_constant__ GridAdjArgs A)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     const GridArgs &G = A.g;
@@ -1489,14 +1487,15 @@ __global__ void __launch_bounds__(GADJ_BLOCK) grid_adjoint_kernel(const __grid_c
 
     const int lane = threadIdx.x & 31;
     const float INF = __int_as_float(0x7f800000);
-    // null scores: inside the box around the beam axis, this CTA's copy of
-    // the voxel sums (many CTAs adding to the same voxels there at once
-    // serialise in L2; the copies spread them)
+    // inside the box around the beam axis, this CTA's copy of the voxel sums:
+    // additions to one address follow each other in L2 at a few per
+    // microsecond, and every photon's first collisions lie there (the copies
+    // spread them; the beam's own row of first flights has copies of its own)
     const size_t cpb = (size_t)(blockIdx.x % (unsigned)A.copies) * A.bstride;
     double *gs = A.gsum, *s1c = A.s1, *bgs = A.bgs + cpb, *bs1 = A.bs1 + cpb;
     auto slot = [&](double *main, double *box, int ix, int iy, int iz, size_t v) -> double * {
         const unsigned by = (unsigned)(iy - A.by0), bz = (unsigned)(iz - A.bz0);
-        if (NULLS && by < (unsigned)A.bw && bz < (unsigned)A.bw)
+        if (by < (unsigned)A.bw && bz < (unsigned)A.bw)
             return box + ((size_t)bz * A.bw + by) * G.gx + ix;
         return main + v;
     };
@@ -1529,7 +1528,7 @@ __global__ void __launch_bounds__(GADJ_BLOCK) grid_adjoint_kernel(const __grid_c
             if (!alive && mine < R.limit) start(mine);
             if (!__any_sync(FULL, alive)) break;
         }
-        int nseg = 0;          // stretches of the flight this lane queued this round
+        int nseg = 0;          // pieces of the flight this lane queued this round
 
         if (alive && ncoll == 0xFFFFFFFFu) {
             // start (or restart) the photon's pass at the entry point
@@ -1606,29 +1605,36 @@ __global__ void __launch_bounds__(GADJ_BLOCK) grid_adjoint_kernel(const __grid_c
                                 // first flight, along +x from the entry point in this
                                 // voxel row: the voxels before ix by the row suffix
                                 gv = fmaf(coef, fmaxf(fmaf(-(float)ix, G.vx, rx), 0.f), gv);
-                                atomicAdd(&A.ex[v], widen(coef));
+                                double *ex = iy == G.gy / 2 && iz == G.gz / 2
+                                                 ? A.exr + (size_t)(blockIdx.x % (unsigned)kRowCopies) * G.gx + ix
+                                                 : A.ex + v;
+                                atomicAdd(ex, widen(coef));
                             } else {
                                 const float ex = rx - px, ey = ry - py, ez = rz - pz;
-                                const float len = sqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez)));
+                                float len = sqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez)));
                                 const Cross X = axis_cross(px, dx, idx, 0.f, G.vx, G.inv_vx, G.gx, len);
                                 const Cross Y = axis_cross(py, dy, idy, -C.hy, G.vy, G.inv_vy, G.gy, len);
                                 const Cross Z = axis_cross(pz, dz, idz, -C.hz, G.vz, G.inv_vz, G.gz, len);
-                                // partition axis: the one crossed most; then the other two
-                                const int pa = (X.n >= Y.n && X.n >= Z.n) ? 0 : (Y.n >= Z.n ? 1 : 2);
-                                const Cross &A0 = pa == 0 ? X : (pa == 1 ? Y : Z);
-                                const Cross &B0 = pa == 0 ? Y : X;
-                                const Cross &C0 = pa == 2 ? Y : Z;
-                                const int ab = pa == 0 ? 1 : 0, ac = pa == 2 ? 1 : 2;
+                                // an axis whose interior planes are all crossed: the wall beyond
+                                // them lies at the flight's end or after it, which rounding must
+                                // not turn round (the sliver is below the position's rounding)
+                                len = fminf(len, fminf(cross_at(X.t0, X.dl, X.n),
+                                                       fminf(cross_at(Y.t0, Y.dl, Y.n), cross_at(Z.t0, Z.dl, Z.n))));
                                 float *q = s_seg + lane;
                                 int *qi = reinterpret_cast<int *>(q);
-                                q[0] = A0.t0; q[32] = B0.t0; q[64] = C0.t0;
-                                q[96] = A0.dl; q[128] = B0.dl; q[160] = C0.dl;
-                                qi[192] = A0.n | (pa << 16) | ((A0.up ? 0 : 1) << 18);
-                                qi[224] = B0.n | (ab << 16) | ((B0.up ? 0 : 1) << 18);
-                                qi[256] = C0.n | (ac << 16) | ((C0.up ? 0 : 1) << 18);
+                                q[0] = X.t0; q[32] = X.dl; qi[64] = X.n | (X.up ? 0 : 1 << 16);
+                                q[96] = Y.t0; q[128] = Y.dl; qi[160] = Y.n | (Y.up ? 0 : 1 << 16);
+                                q[192] = Z.t0; q[224] = Z.dl; qi[256] = Z.n | (Z.up ? 0 : 1 << 16);
                                 q[288] = len; q[320] = coef;
-                                qi[352] = (Z.i0 * G.gy + Y.i0) * G.gx + X.i0;
-                                nseg = A0.n + 1;
+                                // a flight inside the box (both ends: it is convex) adds to this
+                                // CTA's copy of it
+                                const unsigned y0 = (unsigned)(Y.i0 - A.by0), z0 = (unsigned)(Z.i0 - A.bz0);
+                                const unsigned y1 = y0 + (unsigned)(Y.up ? Y.n : -Y.n);
+                                const unsigned z1 = z0 + (unsigned)(Z.up ? Z.n : -Z.n);
+                                const bool box = max(max(y0, y1), max(z0, z1)) < (unsigned)A.bw;
+                                qi[352] = (box ? (int)(z0 * A.bw + y0) : Z.i0 * G.gy + Y.i0) * G.gx + X.i0;
+                                if (box) qi[64] |= 1 << 17;
+                                nseg = X.n + Y.n + Z.n + 1;
                             }
                         }
                         if (gv != 0.f) atomicAdd(slot(gs, bgs, ix, iy, iz, v), widen(gv));
@@ -1663,29 +1669,37 @@ __global__ void __launch_bounds__(GADJ_BLOCK) grid_adjoint_kernel(const __grid_c
                 alive = false;
             }
         }
-        // the warp rasterises its queued flights together, one stretch between
-        // partition-axis crossings per lane: the stretches of all flights are
-        // numbered in lane order and handed out 32 at a time, each lane
-        // finding its flight by a search over the exclusive prefix sums
-        if (!NULLS && __any_sync(FULL, nseg != 0)) {
-            __syncwarp();
-            int incl = nseg;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(FULL, incl, o);
-                if (lane >= o) incl += t;
-            }
-            const int excl = incl - nseg;
-            const int total = __shfl_sync(FULL, incl, 31);
-            for (int base = 0; base < total; base += 32) {
-                const int g = base + lane;
-                int q = 0, eq = 0;    // last lane whose flight starts at or before g
-                for (int st = 16; st > 0; st >>= 1) {
-                    const int e = __shfl_sync(FULL, excl, q + st);
-                    if (e <= g) { q += st; eq = e; }
+        // the warp rasterises its queued flights together, each cut into units
+        // of about K pieces, K such that there are at most 32 units for up to
+        // 16 flights; each lane finds its unit's flight by a search over the
+        // exclusive prefix sums
+        if (!NULLS) {
+            const unsigned queued = __ballot_sync(FULL, nseg != 0);
+            if (queued) {
+                __syncwarp();
+                const int total = (int)__reduce_add_sync(FULL, (unsigned)nseg);
+                const int room = max(16, 32 - __popc(queued));
+                const float per_unit = fmaxf((float)total * rcp_approx((float)room), 1.f);
+                const int units = nseg ? __float2int_ru((float)nseg * rcp_approx(per_unit)) : 0;
+                int incl = units;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int t = __shfl_up_sync(FULL, incl, o);
+                    if (lane >= o) incl += t;
                 }
-                if (g < total) raster_unit(G, gs, s_seg, q, g - eq);
+                const int excl = incl - units;
+                const int n_units = __shfl_sync(FULL, incl, 31);
+                for (int base = 0; base < n_units; base += 32) {
+                    const int g = base + lane;
+                    int q = 0, eq = 0;    // last lane whose flight starts at or before g
+                    for (int st = 16; st > 0; st >>= 1) {
+                        const int e = __shfl_sync(FULL, excl, q + st);
+                        if (e <= g) { q += st; eq = e; }
+                    }
+                    const int of = __shfl_sync(FULL, units, q);
+                    if (g < n_units) raster_unit(A, bgs, s_seg, q, g - eq, of);
+                }
+                __syncwarp();
             }
-            __syncwarp();
         }
     }
     // fixed-order block reduction of the value
@@ -2239,12 +2253,10 @@ cudaError_t launch_grid_adjoint_one(const GridAdjArgs &a, int rows, double *valu
     if (grid > rows) grid = rows;
     kern<<<(unsigned)grid, GADJ_BLOCK, smem, st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (NULLS) {
-        e = launch_box_merge(a.gsum, a.s1, a.bgs, a.bs1, a.copies, a.nbox, a.bstride, a.g.gx, a.g.gy, a.by0, a.bz0,
-                             a.bw, st);
-        if (e != cudaSuccess) return e;
-    }
-    e = launch_gradient_fold(a.gsum, a.s1, NULLS ? nullptr : a.ex, a.grad, a.g.gx, a.g.gy, a.g.gz, (double)a.k_ext,
+    e = launch_box_merge(a.gsum, a.s1, a.bgs, a.bs1, a.copies, a.nbox, a.bstride, a.g.gx, a.g.gy, a.by0, a.bz0, a.bw,
+                         st);
+    if (e != cudaSuccess) return e;
+    e = launch_gradient_fold(a.gsum, a.s1, NULLS ? nullptr : a.ex, NULLS ? nullptr : a.exr, a.grad, a.g.gx, a.g.gy, a.g.gz, (double)a.k_ext,
                              (double)a.g.vx, (double)a.g.vy, st);
     if (e != cudaSuccess) return e;
     adjoint_reduce<<<1, RED_BLOCK, 0, st>>>(a.partials, (int)grid, 1, value);
