@@ -1365,10 +1365,15 @@ __global__ void __launch_bounds__(1024) grid_kernel(const __grid_constant__ Grid
 // double-precision pipe, a small fraction of the single-precision rate,
 // is not used on this path.
 constexpr int GADJ_BLOCK = 256;
-// per-warp queue of flights to rasterise, one column per lane: for x, y and z
-// the first crossing distance, the spacing of the plane crossings and the count
-// with the direction; then the length, the coefficient and the start voxel
-constexpr int GADJ_SEG = 12;
+// per-warp queue of flights to rasterise: columns of start point, direction,
+// length (negative: inside the box around the beam axis) and coefficient, and
+// the count in the last word. A pass adds at most 32 flights; a warp
+// rasterises once it has 16 (a pass queues about four: fewer, larger rounds).
+constexpr int GADJ_SEG = 8;
+constexpr int GADJ_COLS = 47;
+constexpr int GADJ_FLUSH = GADJ_COLS - 32 + 1;
+constexpr int GADJ_QUEUE = 384;   // words per warp
+static_assert(GADJ_SEG * GADJ_COLS < GADJ_QUEUE, "the count needs a word");
 
 // float -> double by moving the bit fields, on the integer pipe (GB300's
 // double-precision pipe, which converts, takes 2 lanes per clock and SM):
@@ -1397,41 +1402,13 @@ __device__ __forceinline__ float cross_at(float t0, float dl, int j)
     return fmaxf(fmaf((float)j, dl, t0), 0.f);
 }
 
-// One axis of a flight of length len from p along d (1/d = id): start voxel
-// i0, first crossing t0, spacing dl, and n, the interior planes crossed at
-// distances below len.
-struct Cross {
-    float t0, dl;
-    int i0, n;
-    bool up;
-};
-
-// The crossings among 0 .. n-1 at distances < t (LE: <= t), idl about 1 / dl.
-// The product is off by less than one crossing (2^-21 of at most 4096), so one
-// step mends it.
-template <bool LE>
+// The crossings among 0 .. n-1 at distances <= t, idl about 1 / dl. The product
+// is off by less than one crossing (2^-21 of at most 4096), so one step mends it.
 __device__ __forceinline__ int count_to(float t0, float dl, float idl, int n, float t)
 {
     int c = min(max(__float2int_rd((t - t0) * idl) + 1, 0), n);
-    const float below = cross_at(t0, dl, c - 1), above = cross_at(t0, dl, c);
-    if (c > 0 && !(LE ? below <= t : below < t)) --c;
-    else if (c < n && (LE ? above <= t : above < t)) ++c;
-    return c;
-}
-
-__device__ __forceinline__ Cross axis_cross(float p, float d, float id, float lo, float v, float iv, int g,
-                                            float len)
-{
-    Cross c;
-    c.i0 = min(max(__float2int_rd((p - lo) * iv), 0), g - 1);
-    c.up = d > 0.f;
-    c.t0 = __int_as_float(0x7f800000);
-    c.dl = 1.f;
-    c.n = 0;
-    if (!(fabsf(id) < __int_as_float(0x7f800000))) return c;   // no motion along this axis: no crossing
-    c.t0 = (fmaf((float)(c.up ? c.i0 + 1 : c.i0), v, lo) - p) * id;
-    c.dl = v * fabsf(id);
-    c.n = count_to<false>(c.t0, c.dl, fabsf(d) * iv, c.up ? g - 1 - c.i0 : c.i0, len);
+    if (c > 0 && !(cross_at(t0, dl, c - 1) <= t)) --c;
+    else if (c < n && cross_at(t0, dl, c) <= t) ++c;
     return c;
 }
 
@@ -1440,31 +1417,45 @@ __device__ __forceinline__ Cross axis_cross(float p, float d, float id, float lo
 // unit's stretch (the flight's own end closes the last); grad[voxel] += coef *
 // length of each. Crossings are evenly spaced on every axis, so the units of a
 // flight hold the same number of pieces within a few, and a piece belongs to
-// one unit whole. Axes crossed at the same distance advance together. No
-// crossing past an axis's count lies before the flight's end (see the queue).
+// one unit whole. Axes crossed at the same distance advance together. Each lane
+// sets its flight's axes up itself (first crossing, spacing), which with 30
+// lanes of a warp costs as much as it would with the few that queued a flight.
 __device__ __forceinline__ void raster_unit(const GridAdjArgs &A, double *bgs, const float *s_seg, int q, int u,
                                             int units)
 {
     const GridArgs &G = A.g;
     const float *f = s_seg + q;
-    const int *fi = reinterpret_cast<const int *>(f);
-    const float coef = f[320];
-    const bool last = u == units - 1, box = fi[64] >> 17;
+    const float coef = f[7 * GADJ_COLS];
+    const bool last = u == units - 1, box = f[6 * GADJ_COLS] < 0.f;
     double *grad = box ? bgs : A.gsum;
     const int span = box ? (int)A.nbox : G.gx * G.gy * G.gz;
-    const float step = f[288] * rcp_approx((float)units);
-    const float t0 = (float)u * step, t1 = last ? f[288] : (float)(u + 1) * step;
-    int v = fi[352];
-    float t = 0.f, next[3], dl[3], first[3], j[3];
-    int st[3];
+    float len = fabsf(f[6 * GADJ_COLS]);
+    const float lo[3] = {0.f, -G.c.hy, -G.c.hz}, vs[3] = {G.vx, G.vy, G.vz}, iv[3] = {G.inv_vx, G.inv_vy, G.inv_vz};
+    const int g[3] = {G.gx, G.gy, G.gz}, off[3] = {0, box ? A.by0 : 0, box ? A.bz0 : 0};
+    float next[3], dl[3], first[3], j[3];
+    int st[3], lim[3], v = 0;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        first[a] = f[96 * a];
-        dl[a] = f[96 * a + 32];
-        const int w = fi[96 * a + 64];
+        const float p = f[a * GADJ_COLS], d = f[(3 + a) * GADJ_COLS], id = mc_div_n(1.0f, d);
+        const bool up = d > 0.f, moves = fabsf(id) < __int_as_float(0x7f800000);
+        const int i0 = min(max(__float2int_rd((p - lo[a]) * iv[a]), 0), g[a] - 1);
+        // no motion along an axis: its crossings are infinitely far
+        first[a] = moves ? (fmaf((float)(up ? i0 + 1 : i0), vs[a], lo[a]) - p) * id : __int_as_float(0x7f800000);
+        dl[a] = moves ? vs[a] * fabsf(id) : 1.f;
+        lim[a] = up ? g[a] - 1 - i0 : i0;       // interior planes ahead
+        // the wall beyond them lies at the flight's end or after it, which
+        // rounding must not turn round (the sliver is below the position's own)
+        len = fminf(len, cross_at(first[a], dl[a], lim[a]));
         st[a] = a == 0 ? 1 : (a == 1 ? G.gx : G.gx * (box ? A.bw : G.gy));
-        if ((w >> 16) & 1) st[a] = -st[a];
-        const int c = u ? count_to<true>(first[a], dl[a], rcp_approx(dl[a]), w & 0xFFFF, t0) : 0;
+        v += (i0 - off[a]) * st[a];
+        if (!up) st[a] = -st[a];
+    }
+    const float step = len * rcp_approx((float)units);
+    const float t0 = (float)u * step, t1 = last ? len : (float)(u + 1) * step;
+    float t = 0.f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int c = u ? count_to(first[a], dl[a], rcp_approx(dl[a]), lim[a], t0) : 0;
         if (c > 0) t = fmaxf(t, cross_at(first[a], dl[a], c - 1));
         v += c * st[a];
         j[a] = (float)c;   // below 4096: the next distance is one FMA
@@ -1486,6 +1477,47 @@ __device__ __forceinline__ void raster_unit(const GridAdjArgs &A, double *bgs, c
     if (last && t1 > t) atomicAdd(&grad[chk(v, span, G.c.error)], widen(coef * (t1 - t)));
 }
 
+// The warp rasterises the queue's `cnt` flights together, up to 32 at a time:
+// each is cut into units of about K pieces, K such that there are at most 32
+// units, and each lane finds its unit's flight by a search over the exclusive
+// prefix sums.
+__device__ __forceinline__ void raster_queue(const GridAdjArgs &A, double *bgs, const float *s_seg, int cnt)
+{
+    const GridArgs &G = A.g;
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    for (int q0 = 0; q0 < cnt; q0 += 32) {
+        const float *f = s_seg + q0 + lane;
+        const int flights = min(cnt - q0, 32);
+        float pieces = 0.f;
+        if (lane < flights)
+            pieces = fabsf(f[6 * GADJ_COLS]) * (fabsf(f[3 * GADJ_COLS]) * G.inv_vx + fabsf(f[4 * GADJ_COLS]) * G.inv_vy +
+                                                fabsf(f[5 * GADJ_COLS]) * G.inv_vz) + 1.f;
+        float total = pieces;
+        for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(FULL, total, o);
+        const float per_unit = fmaxf(total * rcp_approx((float)max(16, 32 - flights)), 1.f);
+        const int units = __float2int_ru(pieces * rcp_approx(per_unit));
+        int incl = units;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += t;
+        }
+        const int excl = incl - units;
+        const int n_units = __shfl_sync(FULL, incl, 31);
+        for (int base = 0; base < n_units; base += 32) {
+            const int g = base + lane;
+            int q = 0, eq = 0;    // last flight whose units start at or before g
+            for (int st = 16; st > 0; st >>= 1) {
+                const int e = __shfl_sync(FULL, excl, q + st);
+                if (e <= g) { q += st; eq = e; }
+            }
+            const int of = __shfl_sync(FULL, units, q);
+            if (g < n_units) raster_unit(A, bgs, s_seg, q0 + q, g - eq, of);
+        }
+    }
+    __syncwarp();
+}
+
 // NULLS: the flights' transmission is scored at the null collisions of
 // delta tracking instead of integrated along each flight. Against majorants
 // scaled by maj_scale > 1 (so mubar > mu_ext in every voxel) a null
@@ -1505,9 +1537,11 @@ __global__ void __launch_bounds__(GADJ_BLOCK, NULLS ? 0 : 4) grid_adjoint_kernel
     float *s_maj = reinterpret_cast<float *>(smem + tb);
     unsigned long long *s_bar = reinterpret_cast<unsigned long long *>(smem + tb + C.extra_bytes);
     double *s_red = reinterpret_cast<double *>(s_bar + 2);
-    // per-warp queue of flight segments to rasterise: (p, d, 1/d, length, coef)
-    float *s_seg = reinterpret_cast<float *>(s_red + GADJ_BLOCK / 32) + (threadIdx.x & ~31u) * GADJ_SEG;
-    // (column f of lane q at s_seg[32 f + q])
+    // this warp's queue of flights to rasterise
+    float *s_seg = reinterpret_cast<float *>(s_red + GADJ_BLOCK / 32) + (threadIdx.x >> 5) * GADJ_QUEUE;
+    int *s_cnt = reinterpret_cast<int *>(s_seg) + GADJ_QUEUE - 1;
+    if ((threadIdx.x & 31) == 0) *s_cnt = 0;   // seen by the warp after the barriers below
+    // (word f of column q at s_seg[GADJ_COLS f + q])
     Smem S = carve<MC_PHASE_HG, false>(smem, C);
     S.table = smem;
     if (threadIdx.x == 0) mbar_init(s_bar);
@@ -1566,7 +1600,6 @@ __global__ void __launch_bounds__(GADJ_BLOCK, NULLS ? 0 : 4) grid_adjoint_kernel
             if (!alive && mine < R.limit) start(mine);
             if (!__any_sync(FULL, alive)) break;
         }
-        int nseg = 0;          // pieces of the flight this lane queued this round
 
         if (alive && ncoll == 0xFFFFFFFFu) {
             // start (or restart) the photon's pass at the entry point
@@ -1649,30 +1682,18 @@ __global__ void __launch_bounds__(GADJ_BLOCK, NULLS ? 0 : 4) grid_adjoint_kernel
                                 atomicAdd(ex, widen(coef));
                             } else {
                                 const float ex = rx - px, ey = ry - py, ez = rz - pz;
-                                float len = sqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez)));
-                                const Cross X = axis_cross(px, dx, idx, 0.f, G.vx, G.inv_vx, G.gx, len);
-                                const Cross Y = axis_cross(py, dy, idy, -C.hy, G.vy, G.inv_vy, G.gy, len);
-                                const Cross Z = axis_cross(pz, dz, idz, -C.hz, G.vz, G.inv_vz, G.gz, len);
-                                // an axis whose interior planes are all crossed: the wall beyond
-                                // them lies at the flight's end or after it, which rounding must
-                                // not turn round (the sliver is below the position's rounding)
-                                len = fminf(len, fminf(cross_at(X.t0, X.dl, X.n),
-                                                       fminf(cross_at(Y.t0, Y.dl, Y.n), cross_at(Z.t0, Z.dl, Z.n))));
-                                float *q = s_seg + lane;
-                                int *qi = reinterpret_cast<int *>(q);
-                                q[0] = X.t0; q[32] = X.dl; qi[64] = X.n | (X.up ? 0 : 1 << 16);
-                                q[96] = Y.t0; q[128] = Y.dl; qi[160] = Y.n | (Y.up ? 0 : 1 << 16);
-                                q[192] = Z.t0; q[224] = Z.dl; qi[256] = Z.n | (Z.up ? 0 : 1 << 16);
-                                q[288] = len; q[320] = coef;
-                                // a flight inside the box (both ends: it is convex) adds to this
-                                // CTA's copy of it
-                                const unsigned y0 = (unsigned)(Y.i0 - A.by0), z0 = (unsigned)(Z.i0 - A.bz0);
-                                const unsigned y1 = y0 + (unsigned)(Y.up ? Y.n : -Y.n);
-                                const unsigned z1 = z0 + (unsigned)(Z.up ? Z.n : -Z.n);
-                                const bool box = max(max(y0, y1), max(z0, z1)) < (unsigned)A.bw;
-                                qi[352] = (box ? (int)(z0 * A.bw + y0) : Z.i0 * G.gy + Y.i0) * G.gx + X.i0;
-                                if (box) qi[64] |= 1 << 17;
-                                nseg = X.n + Y.n + Z.n + 1;
+                                const float len = sqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez)));
+                                // inside the box by a voxel at both ends (it is convex)?
+                                const unsigned y0 = (unsigned)(centred_cell(py, G.inv_vy, 0.5f * (float)G.gy, G.gy) -
+                                                               A.by0 - 1), y1 = (unsigned)(iy - A.by0 - 1);
+                                const unsigned z0 = (unsigned)(centred_cell(pz, G.inv_vz, 0.5f * (float)G.gz, G.gz) -
+                                                               A.bz0 - 1), z1 = (unsigned)(iz - A.bz0 - 1);
+                                const bool box = (int)max(max(y0, y1), max(z0, z1)) >= 0 &&
+                                                 (int)max(max(y0, y1), max(z0, z1)) < A.bw - 2;
+                                float *q = s_seg + atomicAdd(s_cnt, 1);
+                                q[0] = px; q[GADJ_COLS] = py; q[2 * GADJ_COLS] = pz;
+                                q[3 * GADJ_COLS] = dx; q[4 * GADJ_COLS] = dy; q[5 * GADJ_COLS] = dz;
+                                q[6 * GADJ_COLS] = box ? -len : len; q[7 * GADJ_COLS] = coef;
                             }
                         }
                         if (gv != 0.f) atomicAdd(slot(gs, bgs, ix, iy, iz, v), widen(gv));
@@ -1707,38 +1728,19 @@ __global__ void __launch_bounds__(GADJ_BLOCK, NULLS ? 0 : 4) grid_adjoint_kernel
                 alive = false;
             }
         }
-        // the warp rasterises its queued flights together, each cut into units
-        // of about K pieces, K such that there are at most 32 units for up to
-        // 16 flights; each lane finds its unit's flight by a search over the
-        // exclusive prefix sums
         if (!NULLS) {
-            const unsigned queued = __ballot_sync(FULL, nseg != 0);
-            if (queued) {
-                __syncwarp();
-                const int total = (int)__reduce_add_sync(FULL, (unsigned)nseg);
-                const int room = max(16, 32 - __popc(queued));
-                const float per_unit = fmaxf((float)total * rcp_approx((float)room), 1.f);
-                const int units = nseg ? __float2int_ru((float)nseg * rcp_approx(per_unit)) : 0;
-                int incl = units;
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int t = __shfl_up_sync(FULL, incl, o);
-                    if (lane >= o) incl += t;
-                }
-                const int excl = incl - units;
-                const int n_units = __shfl_sync(FULL, incl, 31);
-                for (int base = 0; base < n_units; base += 32) {
-                    const int g = base + lane;
-                    int q = 0, eq = 0;    // last lane whose flight starts at or before g
-                    for (int st = 16; st > 0; st >>= 1) {
-                        const int e = __shfl_sync(FULL, excl, q + st);
-                        if (e <= g) { q += st; eq = e; }
-                    }
-                    const int of = __shfl_sync(FULL, units, q);
-                    if (g < n_units) raster_unit(A, bgs, s_seg, q, g - eq, of);
-                }
+            __syncwarp();
+            const int cnt = __shfl_sync(FULL, *s_cnt, 0);   // one lane's reading: uniform
+            if (cnt >= GADJ_FLUSH) {
+                raster_queue(A, bgs, s_seg, cnt);
+                if (lane == 0) *s_cnt = 0;
                 __syncwarp();
             }
         }
+    }
+    if (!NULLS) {
+        __syncwarp();
+        raster_queue(A, bgs, s_seg, *s_cnt);
     }
     // fixed-order block reduction of the value
     val += __shfl_xor_sync(FULL, val, 16);
@@ -2270,7 +2272,7 @@ cudaError_t launch_grid_one(const GridArgs &a, const LaunchCfg &cfg, size_t smem
 size_t grid_adjoint_smem(const GridAdjArgs &a)
 {
     const size_t tb = (a.g.c.phase_kind != MC_PHASE_HG) ? a.g.c.table_bytes : 0;
-    return tb + a.g.c.extra_bytes + 16 + sizeof(double) * (GADJ_BLOCK / 32) + sizeof(float) * GADJ_BLOCK * GADJ_SEG;
+    return tb + a.g.c.extra_bytes + 16 + sizeof(double) * (GADJ_BLOCK / 32) + sizeof(float) * (GADJ_BLOCK / 32) * GADJ_QUEUE;
 }
 
 template <int PHASE, bool NULLS>
