@@ -762,17 +762,18 @@ mc_status grid_adjoint_common(const mc_grid *g, const void *d_grid_work, const m
     std::memset(&a, 0, sizeof a);
     fill_grid(a.g, g, mx, my, mz, d_grid_work, &m, geom, camera, run, d_error, nullptr, nullptr, nullptr);
     const size_t nb = up(sizeof(double) * n);
-    // s1, gsum (exact: and ex), the box copies of s1 and of gsum (exact: and
-    // the row copies of ex)
+    // s1, gsum, the box copies of s1 and of gsum; exact: the row copies of ex,
+    // then ex itself (not for a pencil beam, whose first flights lie in one row)
     const int bw = std::min(mcx::kBoxWidth, std::min(g->gy, g->gz));
     const size_t bb = up(sizeof(double) * box_voxels(g)), cb = (size_t)mcx::kBoxCopies * bb;
     const size_t rb = up(sizeof(double) * (size_t)mcx::kRowCopies * g->gx);
-    const size_t main = (nulls ? 2 : 3) * nb, region = main + 2 * cb + (nulls ? 0 : rb);
+    const size_t main = 2 * nb, sums = main + 2 * cb + (nulls ? 0 : rb), region = sums + (nulls ? 0 : nb);
+    const bool rows = !nulls && geom->beam_radius > 0.0;
     auto at = [&](size_t off) { return reinterpret_cast<double *>(w + kAlign + off); };
     a.g.counter = reinterpret_cast<unsigned long long *>(w);
     a.s1 = at(0);
     a.gsum = at(nb);
-    a.ex = nulls ? nullptr : at(2 * nb);
+    a.ex = rows ? at(sums) : nullptr;
     a.bs1 = at(main);
     a.bgs = at(main + cb);
     a.exr = nulls ? nullptr : at(main + 2 * cb);
@@ -793,11 +794,12 @@ mc_status grid_adjoint_common(const mc_grid *g, const void *d_grid_work, const m
     // refused before anything is queued when the table and cells do not fit
     const cudaError_t pe = mcx::grid_adjoint_check(a);
     if (pe != cudaSuccess) return pe == cudaErrorInvalidValue ? MC_ERR_ARG : MC_ERR_CUDA;
-    if (fail(cudaMemsetAsync(w, 0, kAlign + region, st)) ||
-        fail(cudaMemsetAsync(d_grad, 0, sizeof(float) * n, st)) ||
-        fail(cudaMemsetAsync(d_value, 0, sizeof(double), st)))
-        return MC_ERR_CUDA;
-    if (run->n_photons == 0) return MC_OK;
+    if (run->n_photons == 0)   // otherwise the fold writes every voxel, the reduction the value
+        return fail(cudaMemsetAsync(d_grad, 0, sizeof(float) * n, st)) ||
+                       fail(cudaMemsetAsync(d_value, 0, sizeof(double), st))
+                   ? MC_ERR_CUDA
+                   : MC_OK;
+    if (fail(cudaMemsetAsync(w, 0, kAlign + (rows ? region : sums), st))) return MC_ERR_CUDA;
     return cuda_status(mcx::launch_grid_adjoint(a, mcx::grid_adjoint_max_grid(), d_value, st));
 }
 }  // namespace

@@ -123,7 +123,7 @@ struct GridAdjArgs {
     // around the beam axis (where many CTAs add at once) are summed in
     // `copies` copies of the box, bstride elements apart, CTA b adding into
     // copy b % copies: bgs for gsum, bs1 for s1; the row suffix of the beam's
-    // own row in kRowCopies rows exr
+    // own row in kRowCopies rows exr (a pencil beam has no other: ex null)
     double *gsum, *s1, *ex, *exr;
     double *bgs, *bs1;
     int copies, by0, bz0, bw;
@@ -177,8 +177,8 @@ cudaError_t grid_adjoint_check(const GridAdjArgs &a);
 
 // grad[v] = gsum[v] + vx * (sum of ex after v in its row along x)
 //           - k_ext vy * (sum of s1 below v in its column along y); gsum is
-// updated in place by the row sums; ex null: no row terms. exr: kRowCopies
-// further rows of ex for the row (gy / 2, gz / 2).
+// updated in place by the row sums. exr: kRowCopies further rows of ex for the
+// row (gy / 2, gz / 2); ex or exr null: none.
 cudaError_t launch_gradient_fold(double *gsum, const double *s1, const double *ex, const double *exr, float *grad,
                                  int gx, int gy, int gz, double k_ext, double vx, double vy, cudaStream_t stream);
 
