@@ -473,9 +473,14 @@ class Engine:
         the previous check; the flags are cleared either way. The word read
         is kept as last_error (0 when nothing was flagged)."""
         st = N.lib().mc_check(C.c_void_p(self.error.data_ptr()), _stream_handle(stream))
-        self.last_error = int(self.error.cpu().numpy()[0]) & 0xFFFFFFFF
+        self._flags("mc_check", st, stream)
+
+    def _flags(self, what, st, stream):
+        # the status of a clean word says what it holds: reading it again is a
+        # copy and a wait of 25 us
+        self.last_error = 0 if st == N.MC_OK else int(self.error.cpu().numpy()[0]) & 0xFFFFFFFF
         _clear_error(self.error, stream)
-        N.check("mc_check", st)
+        N.check(what, st)
 
     def check_within(self, timeout_ms, stream=None):
         """check() with a host-side watchdog: True when the stream finished
@@ -485,9 +490,7 @@ class Engine:
                                      float(timeout_ms))
         if st == N.MC_NOT_READY:
             return False
-        self.last_error = int(self.error.cpu().numpy()[0]) & 0xFFFFFFFF
-        _clear_error(self.error, stream)
-        N.check("mc_check_within", st)
+        self._flags("mc_check_within", st, stream)
         return True
 
     def result(self):
@@ -595,7 +598,9 @@ def _make_camera_image():
                 walk_med = Medium(float(mu_s), float(mu_a), "table", 0.0, wt)
             engine.run(walk_med, n_photons, seed=seed, **kw)
             engine.check()
-            if wt is not None:
+            # rejected weights leave a table that the walk reports; with no
+            # photons there is no walk
+            if wt is not None and not n_photons:
                 wt.check()
             img = engine.image.to(torch.float64) * 2.0 ** -engine.image_frac_bits
             ctx.engine, ctx.med, ctx.n, ctx.seed, ctx.kw = engine, med, n_photons, grad_seed, kw
@@ -611,7 +616,8 @@ def _make_camera_image():
             ctx.engine.check()
             ds, da, dw = ctx.devs
             gw = out[3:].to(dw) if ctx.n_w else None
-            return out[1].to(ds), out[2].to(da), gw, None, None, None, None, None
+            mu = out[1:3] if ds == da == out.device else out[1:3].cpu()   # one copy for both coefficients
+            return mu[0].to(ds), mu[1].to(da), gw, None, None, None, None, None
 
     return CameraImageFn
 
