@@ -421,6 +421,9 @@ mc_status mc_run_batch(int n, const mc_instance *inst, const mc_geometry *geom, 
     return cuda_status(e);
 }
 
+// the adjoint's hat integrals in its workspace
+static size_t hat_bytes() { return up(sizeof(double) * 256 * mcx::kHatParts); }
+
 size_t mc_adjoint_workspace_bytes(int n_phase_w)
 {
     if (n_phase_w < 0 || n_phase_w == 1 || n_phase_w > 256) return 0;
@@ -428,7 +431,7 @@ size_t mc_adjoint_workspace_bytes(int n_phase_w)
     if (rows < 1) return 0;
     // counter, hat integrals, per-CTA partials, and room for the largest
     // reweighted table when there are phase weights
-    return kAlign + up(sizeof(double) * 256) + up(sizeof(double) * (size_t)rows * (3 + n_phase_w)) +
+    return kAlign + hat_bytes() + up(sizeof(double) * (size_t)rows * (3 + n_phase_w)) +
            (n_phase_w > 0 ? up(mc_table_layout(mcx::kMaxWeightedBins, nullptr)) : 0);
 }
 
@@ -479,10 +482,10 @@ mc_status mc_adjoint(const mc_medium *medium, const mc_geometry *geom, const mc_
     const int rows = mcx::adjoint_max_grid();
     a.counter = reinterpret_cast<unsigned long long *>(wk);
     a.z = reinterpret_cast<double *>(wk + kAlign);
-    a.partials = reinterpret_cast<double *>(wk + kAlign + up(sizeof(double) * 256));
+    a.partials = reinterpret_cast<double *>(wk + kAlign + hat_bytes());
     if (d_phase_w) {
         // the walk samples p h_w / Z(w): the table reweighted on the device
-        unsigned char *wt = wk + kAlign + up(sizeof(double) * 256) +
+        unsigned char *wt = wk + kAlign + hat_bytes() +
                             up(sizeof(double) * (size_t)rows * (3 + n_phase_w));
         if ((e = mcx::launch_weighted_table(a.base_table, medium->n_bins, n_phase_w, d_phase_w, wt, d_error,
                                             st)) != cudaSuccess)

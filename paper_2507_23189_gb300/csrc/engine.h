@@ -79,6 +79,7 @@ struct BatchArgs {
 
 // Gradient of L = sum_pix adj[pix] image[pix] for one medium (see adjoint
 // kernel); partials holds one row of 3 + n_w doubles per CTA.
+constexpr int kHatParts = 8;    // CTAs per hat integral
 struct AdjArgs {
     CommonArgs c;
     MediumArgs m;               // m.table: the table the walk samples (reweighted by w if given)
@@ -87,7 +88,7 @@ struct AdjArgs {
     const float *w;             // [n_w] phase weights (nullptr: all 1)
     const unsigned char *base_table;  // the unweighted table (hat integrals Z_k)
     float c_s;                  // 1/mu_s - 1/mu_ext
-    double *z;                  // [n_w] hat integrals of the unweighted table (workspace)
+    double *z;                  // [kHatParts][n_w] parts of the unweighted table's hat integrals (workspace)
     double *partials;           // [grid][3 + n_w]
     unsigned long long *counter;
 };

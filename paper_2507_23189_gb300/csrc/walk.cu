@@ -1788,8 +1788,11 @@ __device__ __forceinline__ int hat_pair(int nw, float mu, float &f)
 }
 
 // Z_k = int_{-1}^{1} p(mu) phi_k(mu) dmu over the table (bins of constant
-// density), exactly, in double precision: CTA k sums the bins of hat k's
-// support, each thread a strided subset in order, then a fixed-order tree.
+// density), exactly, in double precision: CTA (k, part) sums a part of the bins
+// of hat k's support, each thread a strided subset in order, then a fixed-order
+// tree, into z[part][k]. (Nearly all bins lie in the forward hats: one CTA per
+// hat spent 35 us on the last one's 4096 bins at 2 double-precision lanes per
+// clock.)
 __global__ void hat_integrals_kernel(const unsigned char *table, int nw, double *z)
 {
     __shared__ double part[256];
@@ -1800,8 +1803,10 @@ __global__ void hat_integrals_kernel(const unsigned char *table, int nw, double 
     const int n = hd->n_bins, k = blockIdx.x;
     const double h = 2.0 / (nw - 1), inv_h = (nw - 1) / 2.0, c = -1.0 + k * h;
     const double lo = fmax(c - h, -1.0), hi = fmin(c + h, 1.0);
-    const int j0 = max(table_bin(omu, guide, n, (float)lo) - 1, 0);
-    const int j1 = min(table_bin(omu, guide, n, (float)hi) + 1, n - 1);
+    const int first = max(table_bin(omu, guide, n, (float)lo) - 1, 0);
+    const int last = min(table_bin(omu, guide, n, (float)hi) + 1, n - 1);
+    const int per = (last - first + kHatParts) / kHatParts;
+    const int j0 = first + (int)blockIdx.y * per, j1 = min(j0 + per - 1, last);
     double acc = 0.0;
     for (int j = j0 + (int)threadIdx.x; j <= j1; j += blockDim.x) {
         const double a = fmax(1.0 - (double)omu[j], lo), b = fmin(1.0 - (double)omu[j + 1], hi);
@@ -1818,7 +1823,7 @@ __global__ void hat_integrals_kernel(const unsigned char *table, int nw, double 
         if ((int)threadIdx.x < o) part[threadIdx.x] += part[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) z[k] = part[0];
+    if (threadIdx.x == 0) z[(size_t)blockIdx.y * nw + k] = part[0];
 }
 
 constexpr int ADJ_BLOCK = 256;     // threads per CTA without phase weights
@@ -1876,16 +1881,22 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
         if (!bind_table<PHASE>(S, C)) return;
     }
     if (PHASEW) {
-        for (int k = threadIdx.x; k < nw; k += B) s_w[k] = A.w ? A.w[k] : 1.0f;
+        for (int k = threadIdx.x; k < nw; k += B) {
+            s_w[k] = A.w ? A.w[k] : 1.0f;
+            double zk = 0.0;
+            for (int q = 0; q < kHatParts; ++q) zk += A.z[(size_t)q * nw + k];
+            s_z[k] = zk;
+        }
         __syncthreads();
-        if (threadIdx.x == 0) {   // Z(w) = sum_k w_k Z_k, fixed order
+        if (warp == 0) {   // Z(w) = sum_k w_k Z_k, fixed order
             double zw = 0.0;
-            for (int k = 0; k < nw; ++k) zw += (double)s_w[k] * A.z[k];
-            s_red[0] = zw;
+            for (int k = lane; k < nw; k += 32) zw += (double)s_w[k] * s_z[k];
+            for (int o = 16; o > 0; o >>= 1) zw += __shfl_xor_sync(FULL, zw, o);
+            if (lane == 0) s_red[0] = zw;
         }
         __syncthreads();
         const double zw = s_red[0];
-        for (int k = threadIdx.x; k < nw; k += B) s_z[k] = A.z[k] / zw;
+        for (int k = threadIdx.x; k < nw; k += B) s_z[k] = s_z[k] / zw;
     }
     __syncthreads();
     const float c_s = A.c_s;   // 1/mu_s - 1/mu_ext
@@ -2049,12 +2060,16 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
         row[threadIdx.x] = t;
     }
     if (PHASEW) {
+        // hat k's private sums: a compensated single-precision sum, each thread
+        // starting at another column so that a warp's lanes read different
+        // banks. (Double sums over one bank kept the double-precision pipe
+        // busy for 26 of the kernel's 152 us at 1e6 photons and 64 hats.)
         double gzb = 0.0;
         for (int q = 0; q < warps; ++q) gzb += s_red[q * 4 + 3];
         for (int k = threadIdx.x; k < nw; k += B) {
-            double t = 0.0;
-            for (int q = 0; q < B; ++q) t += (double)rows[k * B + q];
-            row[3 + k] = t - s_z[k] * gzb;
+            float sum = 0.f, comp = 0.f;
+            for (int q = 0; q < B; ++q) kahan_add(sum, comp, rows[k * B + ((q + k) & (B - 1))]);
+            row[3 + k] = ((double)sum - (double)comp) - s_z[k] * gzb;
         }
     }
 }
@@ -2497,7 +2512,7 @@ cudaError_t launch_adjoint_one(const AdjArgs &a, int rows, double *out, cudaStre
     if (cap < grid) grid = cap < 1 ? 1 : cap;
     if (grid > rows) grid = rows;
     if (PHASEW) {
-        hat_integrals_kernel<<<a.n_w, 256, 0, st>>>(a.base_table, a.n_w, a.z);
+        hat_integrals_kernel<<<dim3((unsigned)a.n_w, kHatParts), 256, 0, st>>>(a.base_table, a.n_w, a.z);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     kern<<<(unsigned)grid, block, smem, st>>>(a);
