@@ -225,17 +225,7 @@ mc_status run_common(const mc_medium *m, const mc_geometry *g, const mc_camera *
     // refused before anything is queued when the shared-memory plan does not fit
     cudaError_t e = mcx::check_plan(a.c, launch_cfg(r));
     if (e != cudaSuccess) return e == cudaErrorInvalidValue ? MC_ERR_ARG : MC_ERR_CUDA;
-    if (!r->accumulate) {
-        if ((e = cudaMemsetAsync(t->d_image, 0, sizeof(int64_t) * (size_t)c->nx * c->nz, st)))
-            return cuda_status(e);
-        if ((e = cudaMemsetAsync(t->d_radial, 0, sizeof(int64_t) * (size_t)c->n_radial, st)))
-            return cuda_status(e);
-        if ((e = cudaMemsetAsync(t->d_totals, 0, sizeof(int64_t) * MC_N_TOTALS, st)))
-            return cuda_status(e);
-    }
-    if ((e = cudaMemsetAsync(t->d_work, 0, sizeof(unsigned long long), st))) return cuda_status(e);
-    if (r->n_photons == 0) return MC_OK;
-    e = mcx::launch_walk(a, trace != nullptr, launch_cfg(r), st);
+    e = mcx::launch_walk(a, !r->accumulate, trace != nullptr, launch_cfg(r), st);
     return cuda_status(e);
 }
 
@@ -466,9 +456,9 @@ mc_status mc_adjoint(const mc_medium *medium, const mc_geometry *geom, const mc_
     if (work_bytes < need) return MC_ERR_NOMEM;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e;
-    if ((e = cudaMemsetAsync(d_out, 0, sizeof(double) * (3 + n_phase_w), st))) return MC_ERR_CUDA;
+    if (run->n_photons == 0)   // otherwise the reduction writes every output
+        return cuda_status(cudaMemsetAsync(d_out, 0, sizeof(double) * (3 + n_phase_w), st));
     if ((e = cudaMemsetAsync(d_work, 0, sizeof(unsigned long long), st))) return MC_ERR_CUDA;
-    if (run->n_photons == 0) return MC_OK;
     mcx::AdjArgs a;
     std::memset(&a, 0, sizeof a);
     fill_common(a.c, medium, geom, camera, run, d_error, run->n_photons);
@@ -661,22 +651,13 @@ mc_status mc_run_grid(const mc_grid *g, const void *d_grid_work, const mc_medium
     a.c.n_trace = d_trace ? n_trace : 0;
     a.c.n_trace_events = d_trace ? n_events : 0;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const size_t npix = (size_t)camera->nx * camera->nz;
     auto fail = [](cudaError_t x) { return x != cudaSuccess; };
     // refused before anything is queued when the shared-memory plan does not fit
     const cudaError_t pe = mcx::check_plan(a.c, launch_cfg(run));
     if (pe != cudaSuccess) return pe == cudaErrorInvalidValue ? MC_ERR_ARG : MC_ERR_CUDA;
-    if (fail(cudaMemsetAsync(tallies->d_work, 0, sizeof(unsigned long long), st))) return MC_ERR_CUDA;
-    if (!run->accumulate) {
-        if (fail(cudaMemsetAsync(tallies->d_image, 0, sizeof(int64_t) * npix, st)) ||
-            fail(cudaMemsetAsync(tallies->d_radial, 0, sizeof(int64_t) * camera->n_radial, st)) ||
-            fail(cudaMemsetAsync(tallies->d_totals, 0, sizeof(int64_t) * MC_N_TOTALS, st)))
-            return MC_ERR_CUDA;
-    }
     if (d_trace && fail(cudaMemsetAsync(d_trace, 0xFF, sizeof(int32_t) * 12 * (size_t)n_trace * n_events, st)))
         return MC_ERR_CUDA;
-    if (run->n_photons == 0) return MC_OK;
-    return cuda_status(mcx::launch_grid(a, d_trace != nullptr, launch_cfg(run), st));
+    return cuda_status(mcx::launch_grid(a, !run->accumulate, d_trace != nullptr, launch_cfg(run), st));
 }
 
 // Voxels in the gradients' box around the beam axis: all x, the central

@@ -144,9 +144,9 @@ struct LaunchCfg {
                             // shared memory, the rest global
 };
 
-// Launch the walk (or its trace variant) on `stream`. Returns cudaSuccess or
-// the launch error.
-cudaError_t launch_walk(const WalkArgs &a, bool trace, const LaunchCfg &cfg, cudaStream_t stream);
+// Launch the walk (or its trace variant) on `stream`, after clearing the photon
+// counter and, when fresh, the tallies. Returns cudaSuccess or the launch error.
+cudaError_t launch_walk(const WalkArgs &a, bool fresh, bool trace, const LaunchCfg &cfg, cudaStream_t stream);
 // The shared-memory plan of a walk, batch or grid launch without launching
 // anything: cudaErrorInvalidValue when the table, the majorant cells, the
 // radial profile and the totals (with the image tile image_mode 1 asks for)
@@ -162,8 +162,8 @@ cudaError_t launch_batch(const BatchArgs &a, bool fresh, const LaunchCfg &cfg, c
 cudaError_t launch_adjoint(const AdjArgs &a, int partial_rows, double *out, cudaStream_t stream);
 
 // Launch the delta-tracking walk through a prepared grid (trace: records of
-// real events in c.trace).
-cudaError_t launch_grid(const GridArgs &a, bool trace, const LaunchCfg &cfg, cudaStream_t stream);
+// real events in c.trace), clearing as launch_walk does.
+cudaError_t launch_grid(const GridArgs &a, bool fresh, bool trace, const LaunchCfg &cfg, cudaStream_t stream);
 
 // Per-voxel (mu_ext, optical depth above) and per-cell majorants of a grid.
 cudaError_t launch_grid_prepare(const float *density, int gx, int gy, int gz, int bx, int by, int bz,
