@@ -102,12 +102,14 @@ __device__ __forceinline__ float mc_log(float x)   // x normal
     return y * 0.693147180559945309417f;
 #endif
 }
-__device__ __forceinline__ float mc_exp(float x)
+__device__ __forceinline__ float mc_exp(float x)    // results below 2^-126 become 0
 {
 #ifdef MC_STRICT
     return expf(x);
 #else
-    return __expf(x);
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x * 1.44269504088896340736f));
+    return y;
 #endif
 }
 __device__ __forceinline__ float mc_exp2(float x)   // results below 2^-126 become 0
@@ -378,7 +380,7 @@ __device__ __forceinline__ float camera_psr(const MediumArgs &M, const CommonArg
 // half - 1 there, where a pencil beam puts every first collision.
 __device__ __forceinline__ int centred_cell(float r, float inv, float half, int n)
 {
-    return min(max(__float2int_rd(fmaf(r, inv, half)), 0), n - 1);
+    return (int)min(__float2uint_rd(fmaf(r, inv, half)), (unsigned)(n - 1));   // below 0 the conversion gives 0
 }
 
 // Camera pixel of a collision at (rx, rz).
@@ -1885,7 +1887,8 @@ __device__ __forceinline__ void hat_add(float *rows, int nw_stride, const float 
     rows[(k + 1) * nw_stride + threadIdx.x] += u * f;
 }
 
-template <int PHASE, bool PHASEW>
+// UNIT: weights stay 1 (as in walk_loop).
+template <int PHASE, bool PHASEW, bool UNIT>
 __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constant__ AdjArgs A)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -1944,9 +1947,10 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
     // P_tot - P_i is then accurate to ~1e-7 of the photon's total, far
     // below the statistical error of any gradient
     float P = 0.0f, Ptot = 0.0f;
-    // per-thread sums of A_j, A_j dlog/dmu_s, A_j dlog/dmu_a and j A_j as
-    // compensated single-precision pairs
-    float gs_val = 0.f, gc_val = 0.f, gs_s = 0.f, gc_s = 0.f, gs_a = 0.f, gc_a = 0.f, gs_z = 0.f, gc_z = 0.f;
+    // per-thread sums of A_j, X_j = A_j (S_j - l_j) and j A_j as compensated
+    // single-precision pairs: the derivatives are sum X + c_s sum jA (mu_s) and
+    // sum X - sum jA / mu_ext (mu_a), put together once in double
+    float gs_val = 0.f, gc_val = 0.f, gs_x = 0.f, gc_x = 0.f, gs_z = 0.f, gc_z = 0.f;
     // the photon's first ADJ_LIST sampled angles: hat index, fraction, P_i
     // (indexed with compile-time constants only, so they stay in registers)
     int lk[ADJ_LIST];
@@ -1990,7 +1994,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
 
         const uint4 rnd = philox10(make_uint4(pk0, pk1, ev, 0u), M.rk);
         ++ev;
-        const float u0 = u01(rnd.x), u2 = u01(rnd.z), u3 = u01(rnd.w);
+        const float u0 = u01(rnd.x), u2 = u01(rnd.z);
         const float s = -mc_log(u0) * M.inv_mu_ext;
         const float px = fmaf(s, dx, rx), py = fmaf(s, dy, ry), pz = fmaf(s, dz, rz);
         bool end = !((px > 0.f) & (px < C.lx) & (fabsf(py) < C.hy) & (fabsf(pz) < C.hz));
@@ -1998,7 +2002,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
             rx = px; ry = py; rz = pz;
             ++ncoll;
             Ssc += M.inv_mu_ext - s;
-            w = w * M.albedo;
+            if (!UNIT) w = w * M.albedo;
             int nb, ix, iz;
             const float psr = camera_psr<PHASE>(M, C, S, dy, nb);
             const float l = C.hy - ry;
@@ -2007,11 +2011,9 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
             const float Aj = __ldg(&A.adj[pix]) * nee;
             P += Aj;
             if (pass == 1) {
-                const float jj = (float)ncoll;
                 kahan_add(gs_val, gc_val, Aj);
-                kahan_add(gs_s, gc_s, Aj * (Ssc + jj * c_s - l));
-                kahan_add(gs_a, gc_a, Aj * (Ssc - jj * M.inv_mu_ext - l));
-                kahan_add(gs_z, gc_z, jj * Aj);
+                kahan_add(gs_x, gc_x, Aj * (Ssc - l));
+                kahan_add(gs_z, gc_z, (float)ncoll * Aj);
                 if (PHASEW && Aj != 0.0f) {
                     float f;
                     const int k = chk(hat_pair(nw, dy, f), nw - 1, C.error);
@@ -2037,8 +2039,8 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
                 }
                 if (PHASE == MC_PHASE_HG) rotate_hg(dx, dy, dz, om, hg_opu(M, rnd.y), u2);
                 else rotate(dx, dy, dz, om, u2);
-                if (w < C.rr_thr) {
-                    if (u3 < C.rr_surv) w = w * C.inv_rr_surv;
+                if (!UNIT && w < C.rr_thr) {
+                    if (u01(rnd.w) < C.rr_surv) w = w * C.inv_rr_surv;
                     else end = true;
                 }
                 if (!end && ev >= C.max_events) end = true;
@@ -2070,8 +2072,9 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
     }
 
     // -------- reduce: lanes -> warp -> CTA row of partials (fixed order)
-    double g_val = (double)gs_val - (double)gc_val, g_s = (double)gs_s - (double)gc_s;
-    double g_a = (double)gs_a - (double)gc_a, g_z = (double)gs_z - (double)gc_z;
+    const double x = (double)gs_x - (double)gc_x, g_z0 = (double)gs_z - (double)gc_z;
+    double g_val = (double)gs_val - (double)gc_val, g_s = x + (double)c_s * g_z0;
+    double g_a = x - (double)M.inv_mu_ext * g_z0, g_z = g_z0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         g_val += __shfl_xor_sync(FULL, g_val, o);
@@ -2547,10 +2550,10 @@ int adjoint_max_grid()
 }
 
 namespace {
-template <int PHASE, bool PHASEW>
+template <int PHASE, bool PHASEW, bool UNIT>
 cudaError_t launch_adjoint_one(const AdjArgs &a, int rows, double *out, cudaStream_t st)
 {
-    auto kern = adjoint_kernel<PHASE, PHASEW>;
+    auto kern = adjoint_kernel<PHASE, PHASEW, UNIT>;
     const int nw = PHASEW ? a.n_w : 0;
     const int block = PHASEW ? ADJ_BLOCK_W : ADJ_BLOCK;
     const size_t smem = ((PHASE == MC_PHASE_TABLE && !PHASEW) ? a.c.table_bytes : 0) +
@@ -2581,10 +2584,16 @@ cudaError_t launch_adjoint_one(const AdjArgs &a, int rows, double *out, cudaStre
 cudaError_t launch_adjoint(const AdjArgs &a, int rows, double *out, cudaStream_t st)
 {
     if (rows < 1 || a.c.phase_kind == MC_PHASE_PAPER) return cudaErrorInvalidValue;
-    if (a.c.phase_kind == MC_PHASE_TABLE)
-        return a.n_w ? launch_adjoint_one<0, true>(a, rows, out, st) : launch_adjoint_one<0, false>(a, rows, out, st);
-    if (a.n_w) return cudaErrorInvalidValue;
-    return launch_adjoint_one<1, false>(a, rows, out, st);
+    if (a.n_w && a.c.phase_kind != MC_PHASE_TABLE) return cudaErrorInvalidValue;
+    const bool unit = unit_weights(a.c, a.m.albedo);
+    switch ((a.c.phase_kind == MC_PHASE_TABLE ? (a.n_w ? 2 : 0) : 4) + (unit ? 1 : 0)) {
+    case 0: return launch_adjoint_one<MC_PHASE_TABLE, false, false>(a, rows, out, st);
+    case 1: return launch_adjoint_one<MC_PHASE_TABLE, false, true>(a, rows, out, st);
+    case 2: return launch_adjoint_one<MC_PHASE_TABLE, true, false>(a, rows, out, st);
+    case 3: return launch_adjoint_one<MC_PHASE_TABLE, true, true>(a, rows, out, st);
+    case 4: return launch_adjoint_one<MC_PHASE_HG, false, false>(a, rows, out, st);
+    default: return launch_adjoint_one<MC_PHASE_HG, false, true>(a, rows, out, st);
+    }
 }
 
 cudaError_t launch_philox(const uint32_t *ctr, uint64_t n, uint64_t seed, uint32_t *out, cudaStream_t st)

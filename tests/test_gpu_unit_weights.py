@@ -64,3 +64,16 @@ def test_absorbing_media_are_general(gpu, ps_table):
     b.check()
     np.testing.assert_array_equal(b.totals[1].cpu().numpy(), r["raw_totals"])
     assert int(b.totals[0, 3]) == 0
+
+
+@pytest.mark.parametrize("phase,n_w", [("table", 0), ("table", 7), ("table", 200), ("hg", 0)])
+def test_adjoint(gpu, ps_table, phase, n_w):
+    import torch
+    e = gpu.Engine(gpu.Camera(32, 20, 8), gpu.Geometry(45.0, 10.0, 10.0))
+    adj = torch.linspace(0.0, 1.0, 640, device="cuda").view(20, 32)
+    med = _medium(gpu, phase, ps_table)
+    got = [e.adjoint(med, adj, 60_001, n_w=n_w, seed=4, **rr).cpu().numpy() for rr in (UNIT, GENERAL)]
+    e.check()
+    # the same terms in single precision, added in another order: compensated
+    # sums, and private sums of a few terms each over the hats
+    np.testing.assert_allclose(got[0], got[1], rtol=2e-6, atol=2e-6 * np.abs(got[1]).max())
