@@ -750,7 +750,7 @@ __device__ __forceinline__ void walk_loop(const CommonArgs &C, const MediumArgs 
         if (need) {
             const uint32_t mine = P.take(R, need);
             if (!alive && mine < R.limit) start(mine);
-            if (!__any_sync(FULL, alive)) break;
+            if (P.dry && !__any_sync(FULL, alive)) break;
         }
         if (!alive) continue;
 
@@ -1222,7 +1222,7 @@ __device__ __forceinline__ void grid_loop(const GridArgs &G, const Smem &S, cons
         if (need) {
             const uint32_t mine = P.take(R, need);
             if (!alive && mine < R.limit) start(mine);
-            if (!__any_sync(FULL, alive)) break;
+            if (P.dry && !__any_sync(FULL, alive)) break;
         }
         if (!alive) continue;
 
