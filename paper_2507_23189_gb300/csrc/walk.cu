@@ -207,6 +207,36 @@ __device__ __forceinline__ void band_add(uint32_t *cell, unsigned long long *gpi
     if (up) atomicAdd(gpix, (unsigned long long)up << 32);
 }
 
+// One camera contribution vf = weight x 2^image_frac_bits >= 0 into pixel pix:
+// into the band's low words if the pixel lies there, else into global memory.
+// Below 2^32 (the largest float below it is 2^32 - 256) a 32-bit conversion
+// and no high word do, which is nearly every contribution at the bits a run
+// chooses: the 64-bit conversion runs on the double-precision pipe, 2 lanes a
+// clock (walk-hg 230 -> 225 us for 1e6 photons at albedo 0.8, 64 media 733 ->
+// 726 us, the plume's 1e8 photons and unit weights within 1 %). Both round to
+// nearest even, so the tally is the same number either way.
+template <bool SMEM_IMAGE>
+__device__ __forceinline__ void image_add(uint32_t *s_img, const CommonArgs &C, unsigned long long *image,
+                                          int pix, float vf)
+{
+    const unsigned at = (unsigned)(pix - C.band_first);
+    const bool in_band = SMEM_IMAGE && at < (unsigned)C.band_pixels;
+    if (vf < 4294967040.0f) {
+        const uint32_t v = __float2uint_rn(vf);
+        if (in_band) {
+            if (atomicAdd(&s_img[at], v) + v < v) atomicAdd(&image[pix], 1ull << 32);
+        } else {
+            atomicAdd(&image[pix], (unsigned long long)v);
+        }
+    } else if (vf < 4.0e18f) {
+        const long long v = __float2ll_rn(vf);
+        if (in_band) band_add(&s_img[at], &image[pix], v);
+        else atomicAdd(&image[pix], (unsigned long long)v);
+    } else {
+        atomicOr(C.error, (vf == vf) ? MC_EFLAG_OVERFLOW : MC_EFLAG_NUMERIC);
+    }
+}
+
 // mbarrier for the table copies; initialised once per CTA by thread 0.
 __device__ __forceinline__ void mbar_init(unsigned long long *mbar)
 {
@@ -834,14 +864,7 @@ __device__ __forceinline__ void walk_loop(const CommonArgs &C, const MediumArgs 
         const float nee = w * psr * mc_exp2(fmaf(cam_a, ry, cam_b));
         const int pix = camera_pixel_inside(C, rx, rz, ix, iz);   // 0 < rx < lx, |rz| < hz tested above
         const float vf = nee * C.img_scale;
-        if (vf < 4.0e18f) {
-            const long long v = __float2ll_rn(vf);
-            const unsigned at = (unsigned)(pix - C.band_first);
-            if (SMEM_IMAGE && at < (unsigned)C.band_pixels) band_add(&s_img[at], &M.image[pix], v);
-            else atomicAdd(&M.image[pix], (unsigned long long)v);
-        } else {
-            atomicOr(C.error, (vf == vf) ? MC_EFLAG_OVERFLOW : MC_EFLAG_NUMERIC);
-        }
+        image_add<SMEM_IMAGE>(s_img, C, M.image, pix, vf);
 
         if (TRACE) {
             int status = 0;
@@ -1301,14 +1324,7 @@ __device__ __forceinline__ void grid_loop(const GridArgs &G, const Smem &S, cons
         const float nee = w * psr * mc_exp(-fmaf(cell.x, top - ry, cell.y));
         const int pix = camera_pixel(C, rx, rz, pix_x, pix_z);
         const float vf = nee * C.img_scale;
-        if (vf < 4.0e18f) {
-            const long long v = __float2ll_rn(vf);
-            const unsigned at = (unsigned)(pix - C.band_first);
-            if (SMEM_IMAGE && at < (unsigned)C.band_pixels) band_add(&s_img[at], &M.image[pix], v);
-            else atomicAdd(&M.image[pix], (unsigned long long)v);
-        } else {
-            atomicOr(C.error, (vf == vf) ? MC_EFLAG_OVERFLOW : MC_EFLAG_NUMERIC);
-        }
+        image_add<SMEM_IMAGE>(s_img, C, M.image, pix, vf);
         if (TRACE) {
             int status = 0;
             if (ncoll >= C.scatter_cap) {
