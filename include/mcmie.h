@@ -289,8 +289,9 @@ mc_status mc_run_static(const mc_medium *medium, const mc_geometry *geom,
                         uint32_t *d_error, void *stream);
 
 /* Many media in one launch: the CTAs are shared out among the media by
- * estimated photon-steps; a CTA's warps take chunks of item_photons photons
- * of its medium from that medium's counter (0: 128; else 32 .. 2^20), and
+ * estimated photon-steps; a CTA's warps take chunks of at most item_photons
+ * photons (0: 128; else 32 .. 2^20; fewer as the medium's photons run out)
+ * of its medium from that medium's counter, and
  * when the medium's photons are all taken the CTA flushes its tallies into
  * the medium's, joins the medium with most work left per CTA (staging its
  * table in shared memory) and goes on, so the media follow one

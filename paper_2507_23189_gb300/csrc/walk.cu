@@ -212,9 +212,9 @@ __device__ __forceinline__ void band_add(uint32_t *cell, unsigned long long *gpi
 // Below 2^32 (the largest float below it is 2^32 - 256) a 32-bit conversion
 // and no high word do, which is nearly every contribution at the bits a run
 // chooses: the 64-bit conversion runs on the double-precision pipe, 2 lanes a
-// clock (walk-hg 230 -> 225 us for 1e6 photons at albedo 0.8, 64 media 733 ->
-// 726 us, the plume's 1e8 photons and unit weights within 1 %). Both round to
-// nearest even, so the tally is the same number either way.
+// clock (H-G at tau 20 with absorption, 3e6 photons, 230 -> 225 us; 64 media of
+// 2e5 photons 733 -> 726 us; 2e7 photons through the plume 7.86 -> 7.80 ms).
+// Both round to nearest even, so the tally is the same number either way.
 template <bool SMEM_IMAGE>
 __device__ __forceinline__ void image_add(uint32_t *s_img, const CommonArgs &C, unsigned long long *image,
                                           int pix, float vf)
@@ -987,7 +987,8 @@ __device__ __forceinline__ int pick_medium(const BatchArgs &B, int lane)
 // one medium's drain overlaps other media's work: 64 media of 2e5 photons on
 // 128 x 128 images take 0.85 ms a call against 3.87 ms when every CTA went
 // through every medium (the grid then was as large as the largest medium
-// could feed, 49 CTAs); 64 media of 1e6 to 1e8 photons 78.8 against 83.2 ms.
+// could feed, 49 CTAs); 64 media of 1e6 to 1e8 photons 78.8 against 83.2 ms
+// (0.73 and 67.0 ms with the walk as it is now).
 template <int PHASE, bool SMEM_IMAGE, bool UNIT>
 __global__ void __launch_bounds__(1024) batch_kernel(const __grid_constant__ BatchArgs B)
 {
