@@ -1626,7 +1626,11 @@ __global__ void __launch_bounds__(GADJ_BLOCK, NULLS ? 0 : 4) grid_adjoint_kernel
     const LaunchRange R{G.counter, (uint32_t)M.n_photons};
     Pool pool = launch_pool(R);
     bool alive = false;
-    int pass = 0;
+    // 0 in the first pass; in the second the photon's collisions: a flight after
+    // the last of them carries no camera term and is not walked again (5e5
+    // photons, null scores, tau 10: 1007 -> 979 us a step; 2e6 through the plume,
+    // exact lengths: 6.44 -> 6.34 ms)
+    uint32_t total = 0;
     uint32_t pk0 = 0, pk1 = 0, ev = 0, ncoll = 0;
     float rx = 0, ry = 0, rz = 0, dx = 1, dy = 0, dz = 0, w = 1;
     float idx = 1, idy = INF, idz = INF;
@@ -1640,7 +1644,7 @@ __global__ void __launch_bounds__(GADJ_BLOCK, NULLS ? 0 : 4) grid_adjoint_kernel
         const unsigned long long p = M.photon_offset + mine;
         pk0 = (uint32_t)p;
         pk1 = (uint32_t)(p >> 32);
-        pass = 0;
+        total = 0;
         ev = 0;
         ncoll = 0xFFFFFFFFu;
     };
@@ -1677,7 +1681,7 @@ __global__ void __launch_bounds__(GADJ_BLOCK, NULLS ? 0 : 4) grid_adjoint_kernel
         if (!alive) {
             // nothing to walk; still takes part in the warp's rasterisation below
         } else if (ev >= C.max_events) {
-            if (pass == 0) atomicOr(C.error, MC_EFLAG_EVENTS);
+            if (total == 0) atomicOr(C.error, MC_EFLAG_EVENTS);
             end = true;
         } else {
             const uint4 rnd = philox10(make_uint4(pk0, pk1, ev, 0u), M.rk);
@@ -1698,7 +1702,7 @@ __global__ void __launch_bounds__(GADJ_BLOCK, NULLS ? 0 : 4) grid_adjoint_kernel
                 const size_t v = chk((iz * G.gy + iy) * G.gx + ix, G.gx * G.gy * G.gz, C.error);
                 const float2 cell = __ldg(&G.cells[v]);
                 const float acc = mc_div_n(cell.x, mb);   // hardware reciprocal (a few ulp) unless strict
-                if (NULLS && !(u3 < acc) && pass == 1) {
+                if (NULLS && !(u3 < acc) && total != 0) {
                     // null collision: its score times the camera terms after it
                     const float B = Ptot - P;
                     if (B != 0.f) atomicAdd(slot(gs, bgs, ix, iy, iz, v), widen(-B * mc_div_n(A.k_ext, mb - cell.x)));
@@ -1714,7 +1718,7 @@ __global__ void __launch_bounds__(GADJ_BLOCK, NULLS ? 0 : 4) grid_adjoint_kernel
                     const float nee = w * psr * mc_exp(-fmaf(cell.x, top - ry, cell.y));
                     const int pix = camera_pixel(C, rx, rz, pix_x, pix_z);
                     const float Aj = __ldg(&A.adj[pix]) * nee;
-                    if (pass == 1) {
+                    if (total != 0) {
                         const float B = Ptot - P;
                         // column source: this voxel's part directly, the rest by the fold
                         float gv = -A.k_ext * Aj * (top - ry);
@@ -1753,7 +1757,7 @@ __global__ void __launch_bounds__(GADJ_BLOCK, NULLS ? 0 : 4) grid_adjoint_kernel
                     }
                     P += Aj;
                     px = rx; py = ry; pz = rz;
-                    if (ncoll >= C.scatter_cap) {
+                    if (ncoll >= C.scatter_cap || ncoll == total) {
                         end = true;
                     } else {
                         scatter<PHASE>(M, C, S, rnd.y, u2, dx, dy, dz);
@@ -1767,11 +1771,11 @@ __global__ void __launch_bounds__(GADJ_BLOCK, NULLS ? 0 : 4) grid_adjoint_kernel
             }
         }
         if (alive && end) {
-            if (pass == 0) {
+            if (total == 0) {
                 Ptot = P;
                 val += (double)P;
                 if (P != 0.f) {
-                    pass = 1;
+                    total = ncoll;
                     ncoll = 0xFFFFFFFFu;   // replay
                 } else {
                     alive = false;
