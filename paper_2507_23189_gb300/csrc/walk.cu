@@ -1828,9 +1828,9 @@ __global__ void __launch_bounds__(GADJ_BLOCK, NULLS ? 0 : 4) grid_adjoint_kernel
 // S_j = sum over the flights up to j of (1/mu_ext - s_i) (Eq. 15 score),
 // l_j the distance to the camera face, mu_i the sampled polar cosines. The
 // last sum is rearranged as sum_i phi_k(mu_i)/h_w(mu_i) (P_tot - P_i) with
-// P_i = A_1 + .. + A_i, which needs the photon's total P_tot: photons with
-// more angles than the kernel keeps are replayed a second time (same
-// counters). Roulette factors are held fixed.
+// P_i = A_1 + .. + A_i, which needs the photon's total P_tot: a photon with
+// more angles than the kernel keeps is walked a second time from the last of
+// these on (same counters). Roulette factors are held fixed.
 
 // Hat functions: nodes mu_k = -1 + k h, h = 2/(n_w - 1); the two nonzero
 // weights at mu.
@@ -1884,7 +1884,14 @@ __global__ void hat_integrals_kernel(const unsigned char *table, int nw, double 
 
 constexpr int ADJ_BLOCK = 256;     // threads per CTA without phase weights
 constexpr int ADJ_BLOCK_W = 128;   // with phase weights (private accumulators)
-constexpr int ADJ_LIST = 8;        // sampled angles kept per photon before a replay is needed
+// Sampled angles kept per photon. Of a photon with more, the walk is taken up
+// again at the last kept angle (its state is kept too) and ends at the last
+// collision, which carries no later term: 1e7 photons, 64 weights, tau 1 / 5 /
+// 15 375 / 977 / 2336 us -> 364 / 919 / 2035 against a second walk from the
+// entry point to the exit. 6, 5 and 4 angles: 361 / 954 / 2149, 352 / 939 /
+// 2114 and 347 / 969 / 2159 us; more than 8 pass the 80 registers that six
+// CTAs an SM leave.
+constexpr int ADJ_LIST = 8;
 
 // Compensated (Kahan) sum in single precision: s + c carries the running
 // total to about 2^-46 of the summed magnitudes, on the full-rate float pipe
@@ -1961,7 +1968,8 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
     const LaunchRange R{A.counter, (uint32_t)M.n_photons};
     Pool pool = launch_pool(R);
     bool alive = false;
-    int pass = 1, cnt = 0;
+    int pass = 1, cnt = 0;                 // cnt: angles sampled
+    uint32_t total = 0;                    // second pass: the photon's collisions
     uint32_t pk0 = 0, pk1 = 0, ev = 0, ncoll = 0;
     float rx = 0, ry = 0, rz = 0, dx = 1, dy = 0, dz = 0, w = 1, Ssc = 0;
     // the photon's running and total camera terms in single precision:
@@ -1972,12 +1980,15 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
     // single-precision pairs: the derivatives are sum X + c_s sum jA (mu_s) and
     // sum X - sum jA / mu_ext (mu_a), put together once in double
     float gs_val = 0.f, gc_val = 0.f, gs_x = 0.f, gc_x = 0.f, gs_z = 0.f, gc_z = 0.f;
-    // the photon's first ADJ_LIST sampled angles: hat index, fraction, P_i
-    // (indexed with compile-time constants only, so they stay in registers)
-    int lk[ADJ_LIST];
+    // the photon's first ADJ_LIST sampled angles, the last first: hat index (a
+    // byte of lk: at most 256 hats), fraction, P_i (moved along and indexed
+    // with compile-time constants, so they stay in registers)
+    unsigned long long lk = 0;
     float lf[ADJ_LIST], lp[ADJ_LIST];
 #pragma unroll
-    for (int q = 0; q < ADJ_LIST; ++q) { lk[q] = 0; lf[q] = 0.0f; lp[q] = 0.0f; }
+    for (int q = 0; q < ADJ_LIST; ++q) { lf[q] = 0.0f; lp[q] = 0.0f; }
+    // the photon after the list's last angle
+    float kx = 0, ky = 0, kz = 0, kdx = 0, kdy = 0, kdz = 0, kw = 1;
 
     // a lane's next photon (its state is set at the start of a pass)
     auto start = [&](uint32_t mine) {
@@ -1997,7 +2008,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
         }
         if (!alive) continue;
         if (ev == 0) {
-            // (re)start of a pass: the photon enters as in the forward walk
+            // the photon enters as in the forward walk
             rx = 0.f; ry = 0.f; rz = 0.f;
             dx = 1.f; dy = 0.f; dz = 0.f;
             w = 1.f;
@@ -2041,7 +2052,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
                     hat_add(rows, B, s_w, k, f, Aj);
                 }
             }
-            if (ncoll >= C.scatter_cap) {
+            if (ncoll >= C.scatter_cap || (PHASEW && pass == 2 && ncoll == total)) {
                 end = true;
             } else {
                 const float om = sample_omu<PHASE>(M, C, S, rnd.y);
@@ -2049,9 +2060,13 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
                     float f;
                     const int k = chk(hat_pair(nw, 1.0f - om, f), nw - 1, C.error);
                     if (pass == 1) {
+                        if (cnt < ADJ_LIST) {
 #pragma unroll
-                        for (int q = 0; q < ADJ_LIST; ++q)
-                            if (q == cnt) { lk[q] = k; lf[q] = f; lp[q] = P; }
+                            for (int q = ADJ_LIST - 1; q > 0; --q) { lf[q] = lf[q - 1]; lp[q] = lp[q - 1]; }
+                            lk = lk << 8 | (unsigned)k;
+                            lf[0] = f;
+                            lp[0] = P;
+                        }
                         ++cnt;
                     } else {
                         const float coef = Ptot - P;
@@ -2065,30 +2080,41 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
                     else end = true;
                 }
                 if (!end && ev >= C.max_events) end = true;
+                if (PHASEW && pass == 1 && ncoll == ADJ_LIST) {
+                    kx = rx; ky = ry; kz = rz;
+                    kdx = dx; kdy = dy; kdz = dz;
+                    if (!UNIT) kw = w;
+                }
             }
         }
         if (end) {
-            bool replay = false;
             if (PHASEW && pass == 1 && P != 0.0f) {
-                if (cnt <= ADJ_LIST) {
-                    // every sampled angle is in the list: sum_i phi(mu_i) (P_tot - P_i)
+                // the list's angles: phi(mu_i) (P_tot - P_i)
 #pragma unroll
-                    for (int q = 0; q < ADJ_LIST; ++q) {
-                        if (q < cnt) {
-                            const float coef = P - lp[q];
-                            if (coef != 0.0f) hat_add(rows, B, s_w, lk[q], lf[q], coef);
-                        }
+                for (int q = 0; q < ADJ_LIST; ++q) {
+                    if (q < cnt) {
+                        const float coef = P - lp[q];
+                        if (coef != 0.0f) hat_add(rows, B, s_w, (int)(lk >> (8 * q)) & 255, lf[q], coef);
                     }
-                } else {
-                    Ptot = P;   // replay the same photon for its later angles
-                    pass = 2;
-                    replay = true;
                 }
             }
-            if (!replay) alive = false;
-            ev = 0;
-            ncoll = 0;
-            Ssc = 0.0f;
+            if (PHASEW && pass == 1 && P != 0.0f && cnt > ADJ_LIST) {
+                // the later angles: from the list's last on, to the last collision
+                Ptot = P;
+                P = lp[0];
+                pass = 2;
+                total = ncoll;
+                ev = ADJ_LIST;
+                ncoll = ADJ_LIST;
+                rx = kx; ry = ky; rz = kz;
+                dx = kdx; dy = kdy; dz = kdz;
+                if (!UNIT) w = kw;
+            } else {
+                alive = false;
+                ev = 0;
+                ncoll = 0;
+                Ssc = 0.0f;
+            }
         }
     }
 

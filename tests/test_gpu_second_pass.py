@@ -31,3 +31,28 @@ def test_voxel_sums_match_the_homogeneous_gradient(gpu, ps_table, mu_a, kw):
     # the bounds of the same identity without a cap, 1e6 photons
     assert float(value) == pytest.approx(h[0], rel=2e-4)
     assert float(rho) * float(grad.double().sum()) == pytest.approx(mu_s * h[1] + mu_p * h[2], rel=2e-3)
+
+
+@pytest.mark.parametrize("kw", [dict(max_scatter=8), dict(max_scatter=9), dict(max_events=9), dict(max_events=10),
+                                dict(max_scatter=17), {}])
+@pytest.mark.parametrize("n_w,mu_a", [(5, 0.0), (256, 0.0), (64, 0.02)])
+def test_angles_beyond_the_kept_ones(gpu, oracle_mod, ps_table, ps_oracle_table, n_w, mu_a, kw):
+    """Photons around the eight kept angles, at an optical depth where many have
+    more, against the oracle on the same photons (the bounds of the comparison
+    without a cap)."""
+    import torch
+    n, nx, nz = 60_000, 32, 32
+    mu_s = 12.0 / LX - mu_a
+    adj = np.random.default_rng(8).uniform(0, 1, (nz, nx)).astype(np.float32)
+    e = _engine(gpu, nx, nz)
+    got = e.adjoint(gpu.Medium(mu_s, mu_a, "table", 0.0, ps_table), torch.from_numpy(adj), n, n_w=n_w, seed=5,
+                    rr_threshold=0.05, **kw)
+    if "max_events" not in kw:
+        e.check()
+    got = got.cpu().numpy()
+    o = oracle_mod.adjoint(adj.astype(np.float64), n_w, mu_s=mu_s, mu_a=mu_a, table=ps_oracle_table, n_photons=n,
+                           nx=nx, nz=nz, seed=5, rr_threshold=0.05, **kw)
+    g = o["grad"]
+    sig = np.sqrt(np.maximum(o["grad_sq"] - g ** 2 / n, 0))
+    assert got[0] == pytest.approx(o["value"], rel=1e-4)
+    assert np.all(np.abs(got[1:] - g) <= 0.05 * sig + 1e-4 * np.abs(g) + 1e-9)
