@@ -1416,7 +1416,7 @@ __global__ void __launch_bounds__(1024) grid_kernel(const __grid_constant__ Grid
 // precision and summed by double-precision atomics in L2; the SM's own
 // double-precision pipe, a small fraction of the single-precision rate,
 // is not used on this path.
-constexpr int GADJ_BLOCK = 256;
+constexpr int GADJ_MIN_BLOCK = 256, GADJ_MAX_BLOCK = 1024;   // see grid_adjoint_block
 // per-warp queue of flights to rasterise: columns of start point, direction,
 // length (negative: inside the box around the beam axis) and coefficient, and
 // the count in the last word. A pass adds at most 32 flights; a warp
@@ -1579,7 +1579,7 @@ __device__ __forceinline__ void raster_queue(const GridAdjArgs &A, double *bgs, 
 // collision replaces the rasterised flight; both are unbiased estimates of
 // the same gradient.
 template <int PHASE, bool NULLS>
-__global__ void __launch_bounds__(GADJ_BLOCK, NULLS ? 0 : 4) grid_adjoint_kernel(const __grid_constant__ GridAdjArgs A)
+__global__ void __launch_bounds__(GADJ_MAX_BLOCK) grid_adjoint_kernel(const __grid_constant__ GridAdjArgs A)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     const GridArgs &G = A.g;
@@ -1590,7 +1590,7 @@ __global__ void __launch_bounds__(GADJ_BLOCK, NULLS ? 0 : 4) grid_adjoint_kernel
     unsigned long long *s_bar = reinterpret_cast<unsigned long long *>(smem + tb + C.extra_bytes);
     double *s_red = reinterpret_cast<double *>(s_bar + 2);
     // this warp's queue of flights to rasterise
-    float *s_seg = reinterpret_cast<float *>(s_red + GADJ_BLOCK / 32) + (threadIdx.x >> 5) * GADJ_QUEUE;
+    float *s_seg = reinterpret_cast<float *>(s_red + blockDim.x / 32) + (threadIdx.x >> 5) * GADJ_QUEUE;
     int *s_cnt = reinterpret_cast<int *>(s_seg) + GADJ_QUEUE - 1;
     if ((threadIdx.x & 31) == 0) *s_cnt = 0;   // seen by the warp after the barriers below
     // (word f of column q at s_seg[GADJ_COLS f + q])
@@ -2389,29 +2389,63 @@ cudaError_t launch_grid_one(const GridArgs &a, const LaunchCfg &cfg, size_t smem
     return launch_after(kern, dim3(grid), cfg.block, smem, st, a);
 }
 
-size_t grid_adjoint_smem(const GridAdjArgs &a)
+size_t grid_adjoint_smem(const GridAdjArgs &a, int block)
 {
     const size_t tb = (a.g.c.phase_kind != MC_PHASE_HG) ? a.g.c.table_bytes : 0;
-    return tb + a.g.c.extra_bytes + 16 + sizeof(double) * (GADJ_BLOCK / 32) + sizeof(float) * (GADJ_BLOCK / 32) * GADJ_QUEUE;
+    return tb + a.g.c.extra_bytes + 16 + (sizeof(double) + sizeof(float) * GADJ_QUEUE) * (block / 32);
+}
+
+// Threads per CTA of the density gradient: the size that keeps most warps on
+// an SM (1024 threads at the kernel's registers, the table and the majorants in
+// shared memory once per CTA), 512 where several do: 2e6 photons through the
+// plume 5.99 ms with 512 threads, about as long with 1024, 6.34 with 256, whose
+// four copies of the table leave less of L1 to the voxel gathers; 5e5 photons with null scores
+// 963, 969 and 979 us. Few photons: 256, to reach more SMs.
+cudaError_t grid_adjoint_block(const GridAdjArgs &a, int *block)
+{
+    int dev = 0, sms = 0, optin = 0, per_sm = 0;
+    cudaError_t e;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess) return e;
+    const bool few = (a.g.m.n_photons + 31) / 32 < (unsigned long long)sms * (512 / 32);
+    const int order[3] = {few ? 256 : 512, few ? 512 : 1024, few ? 1024 : 256};
+    int best = 0;
+    *block = 0;
+    for (int b : order) {
+        const size_t smem = grid_adjoint_smem(a, b);
+        if (smem > (size_t)optin) continue;
+        const int fit = (int)((size_t)per_sm / (smem + 1024)), regs = 1024 / b;
+        const int warps = (b / 32) * (fit < regs ? fit : regs);
+        if (warps > best) {
+            best = warps;
+            *block = b;
+        }
+    }
+    return *block ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 template <int PHASE, bool NULLS>
 cudaError_t launch_grid_adjoint_one(const GridAdjArgs &a, int rows, double *value, cudaStream_t st)
 {
     auto kern = grid_adjoint_kernel<PHASE, NULLS>;
-    const size_t smem = grid_adjoint_smem(a);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int block = 0;
+    cudaError_t e = grid_adjoint_block(a, &block);
     if (e != cudaSuccess) return e;
+    const size_t smem = grid_adjoint_smem(a, block);
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+        return e;
     int dev = 0, sms = 0, bps = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, GADJ_BLOCK, smem)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, block, smem)) != cudaSuccess) return e;
     if (bps < 1) return cudaErrorInvalidConfiguration;
     long long grid = (long long)sms * bps;
-    const long long cap = (long long)((a.g.m.n_photons + 31) / 32 + GADJ_BLOCK / 32 - 1) / (GADJ_BLOCK / 32);
+    const long long cap = (long long)((a.g.m.n_photons + 31) / 32 + block / 32 - 1) / (block / 32);
     if (cap < grid) grid = cap < 1 ? 1 : cap;
     if (grid > rows) grid = rows;
-    kern<<<(unsigned)grid, GADJ_BLOCK, smem, st>>>(a);
+    kern<<<(unsigned)grid, block, smem, st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     e = launch_box_merge(a.gsum, a.s1, a.bgs, a.bs1, a.copies, a.nbox, a.bstride, a.g.gx, a.g.gy, a.by0, a.bz0, a.bw,
                          st);
@@ -2525,12 +2559,8 @@ cudaError_t launch_grid(const GridArgs &a0, bool fresh, bool trace, const Launch
 
 cudaError_t grid_adjoint_check(const GridAdjArgs &a)
 {
-    int dev = 0, optin = 0;
-    cudaError_t e;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
-        return e;
-    return grid_adjoint_smem(a) <= (size_t)optin ? cudaSuccess : cudaErrorInvalidValue;
+    int block = 0;
+    return grid_adjoint_block(a, &block);
 }
 
 int grid_adjoint_max_grid()
@@ -2538,7 +2568,7 @@ int grid_adjoint_max_grid()
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    return sms * (2048 / GADJ_BLOCK);
+    return sms * (2048 / GADJ_MIN_BLOCK);
 }
 
 cudaError_t launch_grid_adjoint(const GridAdjArgs &a, int rows, double *value, cudaStream_t st)

@@ -33,6 +33,29 @@ def test_voxel_sums_match_the_homogeneous_gradient(gpu, ps_table, mu_a, kw):
     assert float(rho) * float(grad.double().sum()) == pytest.approx(mu_s * h[1] + mu_p * h[2], rel=2e-3)
 
 
+@pytest.mark.parametrize("n_bins,cell", [(64, 4), (8192, 4), (16384, 4), (8192, 1)])
+@pytest.mark.parametrize("n", [50, 3_000, 100_000])
+def test_every_cta_size(gpu, n_bins, cell, n):
+    """Few photons and large tables or many cells take other CTA sizes of the
+    gradient kernel: the same identity."""
+    import torch
+    rho = np.float32(0.15)
+    adj = torch.rand((32, 48), generator=torch.Generator().manual_seed(4))
+    e = _engine(gpu, 48, 32)
+    table = gpu.PhaseTable(n_bins=n_bins)
+    grid = gpu.Grid(torch.full((16, 24, 32), float(rho), device="cuda"), 1.0, 0.8, 0.0, (cell, cell, cell))
+    grid = grid.prepare(gpu.Geometry(LX, 10.0, 10.0))
+    value, grad = e.grid_adjoint(grid, gpu.Medium(1.0, 0.0, "table", 0.0, table), adj, n, seed=9)
+    e.check()
+    mu_s, mu_p = 0.8 * float(rho), (1.0 - 0.8) * float(rho)
+    h = e.adjoint(gpu.Medium(mu_s, mu_p, "table", 0.0, table), adj, n, n_w=0, seed=9).cpu().numpy()
+    e.check()
+    assert float(value) == pytest.approx(h[0], rel=2e-4)
+    # few photons: the sums cancel, so against the terms' own size (the value's)
+    bound = 2e-3 * abs(mu_s * h[1] + mu_p * h[2]) + 1e-3 * abs(h[0])
+    assert abs(float(rho) * float(grad.double().sum()) - (mu_s * h[1] + mu_p * h[2])) <= bound
+
+
 @pytest.mark.parametrize("kw", [dict(max_scatter=8), dict(max_scatter=9), dict(max_events=9), dict(max_events=10),
                                 dict(max_scatter=17), {}])
 @pytest.mark.parametrize("n_w,mu_a", [(5, 0.0), (256, 0.0), (64, 0.02)])
