@@ -1416,16 +1416,22 @@ __global__ void __launch_bounds__(1024) grid_kernel(const __grid_constant__ Grid
 // precision and summed by double-precision atomics in L2; the SM's own
 // double-precision pipe, a small fraction of the single-precision rate,
 // is not used on this path.
-constexpr int GADJ_MIN_BLOCK = 256, GADJ_MAX_BLOCK = 1024;   // see grid_adjoint_block
-// per-warp queue of flights to rasterise: columns of start point, direction,
-// length (negative: inside the box around the beam axis) and coefficient, and
-// the count in the last word. A pass adds at most 32 flights; a warp
-// rasterises once it has 16 (a pass queues about four: fewer, larger rounds).
-constexpr int GADJ_SEG = 8;
-constexpr int GADJ_COLS = 47;
+constexpr int GADJ_MAX_BLOCK = 1024;   // see grid_adjoint_block
+// Per-warp queue of the second pass's collisions after the first, whose terms
+// the warp adds and whose flights it rasterises together: columns of the
+// flight's start, direction, end (x, y, z: the words QEX, QEY, QEZ), its
+// coefficient, and the terms of the collision's voxel and of its camera column
+// above; the count in the last word. A pass adds at most 32; a warp takes them
+// up once it has 24 (a pass queues about four: fewer, larger rounds; the
+// plume's kernel 5.46 ms against 5.55 at 16, 6.07 at 8, 5.62 at 32).
+constexpr int GADJ_SEG = 12;
+constexpr int GADJ_COLS = 55;
 constexpr int GADJ_FLUSH = GADJ_COLS - 32 + 1;
-constexpr int GADJ_QUEUE = 384;   // words per warp
-static_assert(GADJ_SEG * GADJ_COLS < GADJ_QUEUE, "the count needs a word");
+constexpr int GADJ_QUEUE = 662;   // words per warp
+static_assert(GADJ_SEG * GADJ_COLS < GADJ_QUEUE && GADJ_QUEUE % 2 == 0, "the count needs a word");
+constexpr int QEX = 6 * GADJ_COLS, QCOEF = 7 * GADJ_COLS, QEY = 8 * GADJ_COLS, QEZ = 9 * GADJ_COLS,
+              QPOINT = 10 * GADJ_COLS, QCOLUMN = 11 * GADJ_COLS;
+constexpr int QLEN = QEX;         // while it is rasterised: the length, negative inside the box around the beam axis
 
 // float -> double by moving the bit fields, on the integer pipe (GB300's
 // double-precision pipe, which converts, takes 2 lanes per clock and SM):
@@ -1477,11 +1483,11 @@ __device__ __forceinline__ void raster_unit(const GridAdjArgs &A, double *bgs, c
 {
     const GridArgs &G = A.g;
     const float *f = s_seg + q;
-    const float coef = f[7 * GADJ_COLS];
-    const bool last = u == units - 1, box = f[6 * GADJ_COLS] < 0.f;
+    const float coef = f[QCOEF];
+    const bool last = u == units - 1, box = f[QLEN] < 0.f;
     double *grad = box ? bgs : A.gsum;
     const int span = box ? (int)A.nbox : G.gx * G.gy * G.gz;
-    float len = fabsf(f[6 * GADJ_COLS]);
+    float len = fabsf(f[QLEN]);
     const float lo[3] = {0.f, -G.c.hy, -G.c.hz}, vs[3] = {G.vx, G.vy, G.vz}, iv[3] = {G.inv_vx, G.inv_vy, G.inv_vz};
     const int g[3] = {G.gx, G.gy, G.gz}, off[3] = {0, box ? A.by0 : 0, box ? A.bz0 : 0};
     float next[3], dl[3], first[3], j[3];
@@ -1529,25 +1535,56 @@ __device__ __forceinline__ void raster_unit(const GridAdjArgs &A, double *bgs, c
     if (last && t1 > t) atomicAdd(&grad[chk(v, span, G.c.error)], widen(coef * (t1 - t)));
 }
 
-// The warp rasterises the queue's `cnt` flights together, up to 32 at a time:
-// each is cut into units of about K pieces, K such that there are at most 32
-// units, and each lane finds its unit's flight by a search over the exclusive
-// prefix sums.
-__device__ __forceinline__ void raster_queue(const GridAdjArgs &A, double *bgs, const float *s_seg, int cnt)
+// The voxel's element in the sums: inside the box around the beam axis, in this
+// CTA's copy of the box (additions to one address follow each other in L2 at a
+// few per microsecond, and every photon's first collisions lie there).
+__device__ __forceinline__ double *box_slot(const GridAdjArgs &A, double *all, double *box, int ix, int iy, int iz, size_t v)
+{
+    const unsigned by = (unsigned)(iy - A.by0), bz = (unsigned)(iz - A.bz0);
+    if (by < (unsigned)A.bw && bz < (unsigned)A.bw) return box + ((size_t)bz * A.bw + by) * A.g.gx + ix;
+    return all + v;
+}
+
+// The warp takes up the queue's `cnt` collisions together, up to 32 at a time:
+// each lane adds one's terms (added where they arise, by the few lanes of a
+// pass that have one: 5.39e9 instead of 5.25e9 warp-instructions). Then the
+// flights are rasterised, cut into units of about K pieces each, and each lane
+// finds its unit's flight by a search over the exclusive prefix sums. K is such
+// that the units, rounded up by half a unit a flight on average, fill one round
+// of the 32 lanes, or two when there are more flights than leave half of one.
+__device__ __forceinline__ void raster_queue(const GridAdjArgs &A, double *bgs, double *bs1, float *s_seg, int cnt)
 {
     const GridArgs &G = A.g;
     const int lane = threadIdx.x & 31;
     __syncwarp();
     for (int q0 = 0; q0 < cnt; q0 += 32) {
-        const float *f = s_seg + q0 + lane;
+        float *f = s_seg + q0 + lane;
         const int flights = min(cnt - q0, 32);
         float pieces = 0.f;
-        if (lane < flights)
-            pieces = fabsf(f[6 * GADJ_COLS]) * (fabsf(f[3 * GADJ_COLS]) * G.inv_vx + fabsf(f[4 * GADJ_COLS]) * G.inv_vy +
-                                                fabsf(f[5 * GADJ_COLS]) * G.inv_vz) + 1.f;
+        if (lane < flights) {
+            const float px = f[0], py = f[GADJ_COLS], pz = f[2 * GADJ_COLS], rx = f[QEX], ry = f[QEY], rz = f[QEZ];
+            const int ix = min(max(__float2int_rd(rx * G.inv_vx), 0), G.gx - 1);
+            const int iy = centred_cell(ry, G.inv_vy, 0.5f * (float)G.gy, G.gy);
+            const int iz = centred_cell(rz, G.inv_vz, 0.5f * (float)G.gz, G.gz);
+            const size_t v = chk((iz * G.gy + iy) * G.gx + ix, G.gx * G.gy * G.gz, G.c.error);
+            const float gv = f[QPOINT], Aj = f[QCOLUMN];
+            if (gv != 0.f) atomicAdd(box_slot(A, A.gsum, bgs, ix, iy, iz, v), widen(gv));
+            if (Aj != 0.f) atomicAdd(box_slot(A, A.s1, bs1, ix, iy, iz, v), widen(Aj));
+            const float ex = rx - px, ey = ry - py, ez = rz - pz;
+            const float len = sqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez)));
+            // inside the box by a voxel at both ends (it is convex)?
+            const unsigned y0 = (unsigned)(centred_cell(py, G.inv_vy, 0.5f * (float)G.gy, G.gy) - A.by0 - 1);
+            const unsigned z0 = (unsigned)(centred_cell(pz, G.inv_vz, 0.5f * (float)G.gz, G.gz) - A.bz0 - 1);
+            const unsigned y1 = (unsigned)(iy - A.by0 - 1), z1 = (unsigned)(iz - A.bz0 - 1);
+            const int far = (int)max(max(y0, y1), max(z0, z1));
+            f[QLEN] = far >= 0 && far < A.bw - 2 ? -len : len;
+            pieces = len * (fabsf(f[3 * GADJ_COLS]) * G.inv_vx + fabsf(f[4 * GADJ_COLS]) * G.inv_vy +
+                            fabsf(f[5 * GADJ_COLS]) * G.inv_vz) + 1.f;
+        }
+        __syncwarp();
         float total = pieces;
         for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(FULL, total, o);
-        const float per_unit = fmaxf(total * rcp_approx((float)max(16, 32 - flights)), 1.f);
+        const float per_unit = fmaxf(total * rcp_approx((flights > 22 ? 60.f : 28.f) - 0.5f * (float)flights), 1.f);
         const int units = __float2int_ru(pieces * rcp_approx(per_unit));
         int incl = units;
         for (int o = 1; o < 32; o <<= 1) {
@@ -1592,7 +1629,7 @@ __global__ void __launch_bounds__(GADJ_MAX_BLOCK) grid_adjoint_kernel(const __gr
     // this warp's queue of flights to rasterise
     float *s_seg = reinterpret_cast<float *>(s_red + blockDim.x / 32) + (threadIdx.x >> 5) * GADJ_QUEUE;
     int *s_cnt = reinterpret_cast<int *>(s_seg) + GADJ_QUEUE - 1;
-    if ((threadIdx.x & 31) == 0) *s_cnt = 0;   // seen by the warp after the barriers below
+    if (!NULLS && (threadIdx.x & 31) == 0) *s_cnt = 0;   // seen by the warp after the barriers below
     // (word f of column q at s_seg[GADJ_COLS f + q])
     Smem S = carve<MC_PHASE_HG, false>(smem, C);
     S.table = smem;
@@ -1611,18 +1648,10 @@ __global__ void __launch_bounds__(GADJ_MAX_BLOCK) grid_adjoint_kernel(const __gr
 
     const int lane = threadIdx.x & 31;
     const float INF = __int_as_float(0x7f800000);
-    // inside the box around the beam axis, this CTA's copy of the voxel sums:
-    // additions to one address follow each other in L2 at a few per
-    // microsecond, and every photon's first collisions lie there (the copies
-    // spread them; the beam's own row of first flights has copies of its own)
+    // this CTA's copies of the sums near the beam axis (the beam's own row of
+    // first flights has copies of its own)
     const size_t cpb = (size_t)(blockIdx.x % (unsigned)A.copies) * A.bstride;
     double *gs = A.gsum, *s1c = A.s1, *bgs = A.bgs + cpb, *bs1 = A.bs1 + cpb;
-    auto slot = [&](double *main, double *box, int ix, int iy, int iz, size_t v) -> double * {
-        const unsigned by = (unsigned)(iy - A.by0), bz = (unsigned)(iz - A.bz0);
-        if (by < (unsigned)A.bw && bz < (unsigned)A.bw)
-            return box + ((size_t)bz * A.bw + by) * G.gx + ix;
-        return main + v;
-    };
     const LaunchRange R{G.counter, (uint32_t)M.n_photons};
     Pool pool = launch_pool(R);
     bool alive = false;
@@ -1705,7 +1734,7 @@ __global__ void __launch_bounds__(GADJ_MAX_BLOCK) grid_adjoint_kernel(const __gr
                 if (NULLS && !(u3 < acc) && total != 0) {
                     // null collision: its score times the camera terms after it
                     const float B = Ptot - P;
-                    if (B != 0.f) atomicAdd(slot(gs, bgs, ix, iy, iz, v), widen(-B * mc_div_n(A.k_ext, mb - cell.x)));
+                    if (B != 0.f) atomicAdd(box_slot(A, gs, bgs, ix, iy, iz, v), widen(-B * mc_div_n(A.k_ext, mb - cell.x)));
                 }
                 if (u3 < acc) {
                     u3 = mc_div_n(u3, acc);
@@ -1720,6 +1749,7 @@ __global__ void __launch_bounds__(GADJ_MAX_BLOCK) grid_adjoint_kernel(const __gr
                     const float Aj = __ldg(&A.adj[pix]) * nee;
                     if (total != 0) {
                         const float B = Ptot - P;
+                        bool queued = false;
                         // column source: this voxel's part directly, the rest by the fold
                         float gv = -A.k_ext * Aj * (top - ry);
                         if (B != 0.f) {
@@ -1737,23 +1767,18 @@ __global__ void __launch_bounds__(GADJ_MAX_BLOCK) grid_adjoint_kernel(const __gr
                                                  : A.ex + v;
                                 atomicAdd(ex, widen(coef));
                             } else {
-                                const float ex = rx - px, ey = ry - py, ez = rz - pz;
-                                const float len = sqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez)));
-                                // inside the box by a voxel at both ends (it is convex)?
-                                const unsigned y0 = (unsigned)(centred_cell(py, G.inv_vy, 0.5f * (float)G.gy, G.gy) -
-                                                               A.by0 - 1), y1 = (unsigned)(iy - A.by0 - 1);
-                                const unsigned z0 = (unsigned)(centred_cell(pz, G.inv_vz, 0.5f * (float)G.gz, G.gz) -
-                                                               A.bz0 - 1), z1 = (unsigned)(iz - A.bz0 - 1);
-                                const bool box = (int)max(max(y0, y1), max(z0, z1)) >= 0 &&
-                                                 (int)max(max(y0, y1), max(z0, z1)) < A.bw - 2;
                                 float *q = s_seg + atomicAdd(s_cnt, 1);
                                 q[0] = px; q[GADJ_COLS] = py; q[2 * GADJ_COLS] = pz;
                                 q[3 * GADJ_COLS] = dx; q[4 * GADJ_COLS] = dy; q[5 * GADJ_COLS] = dz;
-                                q[6 * GADJ_COLS] = box ? -len : len; q[7 * GADJ_COLS] = coef;
+                                q[QEX] = rx; q[QEY] = ry; q[QEZ] = rz;
+                                q[QCOEF] = coef; q[QPOINT] = gv; q[QCOLUMN] = Aj;
+                                queued = true;
                             }
                         }
-                        if (gv != 0.f) atomicAdd(slot(gs, bgs, ix, iy, iz, v), widen(gv));
-                        if (Aj != 0.f) atomicAdd(slot(s1c, bs1, ix, iy, iz, v), widen(Aj));
+                        if (!queued) {
+                            if (gv != 0.f) atomicAdd(box_slot(A, gs, bgs, ix, iy, iz, v), widen(gv));
+                            if (Aj != 0.f) atomicAdd(box_slot(A, s1c, bs1, ix, iy, iz, v), widen(Aj));
+                        }
                     }
                     P += Aj;
                     px = rx; py = ry; pz = rz;
@@ -1788,7 +1813,7 @@ __global__ void __launch_bounds__(GADJ_MAX_BLOCK) grid_adjoint_kernel(const __gr
             __syncwarp();
             const int cnt = __shfl_sync(FULL, *s_cnt, 0);   // one lane's reading: uniform
             if (cnt >= GADJ_FLUSH) {
-                raster_queue(A, bgs, s_seg, cnt);
+                raster_queue(A, bgs, bs1, s_seg, cnt);
                 if (lane == 0) *s_cnt = 0;
                 __syncwarp();
             }
@@ -1796,7 +1821,7 @@ __global__ void __launch_bounds__(GADJ_MAX_BLOCK) grid_adjoint_kernel(const __gr
     }
     if (!NULLS) {
         __syncwarp();
-        raster_queue(A, bgs, s_seg, *s_cnt);
+        raster_queue(A, bgs, bs1, s_seg, *s_cnt);
     }
     // fixed-order block reduction of the value
     val += __shfl_xor_sync(FULL, val, 16);
@@ -2392,15 +2417,19 @@ cudaError_t launch_grid_one(const GridArgs &a, const LaunchCfg &cfg, size_t smem
 size_t grid_adjoint_smem(const GridAdjArgs &a, int block)
 {
     const size_t tb = (a.g.c.phase_kind != MC_PHASE_HG) ? a.g.c.table_bytes : 0;
-    return tb + a.g.c.extra_bytes + 16 + (sizeof(double) + sizeof(float) * GADJ_QUEUE) * (block / 32);
+    return tb + a.g.c.extra_bytes + 16 + (sizeof(double) + (a.nulls ? 0 : sizeof(float) * GADJ_QUEUE)) * (block / 32);
 }
 
 // Threads per CTA of the density gradient: the size that keeps most warps on
 // an SM (1024 threads at the kernel's registers, the table and the majorants in
 // shared memory once per CTA), 512 where several do: 2e6 photons through the
 // plume 5.99 ms with 512 threads, about as long with 1024, 6.34 with 256, whose
-// four copies of the table leave less of L1 to the voxel gathers; 5e5 photons with null scores
-// 963, 969 and 979 us. Few photons: 256, to reach more SMs.
+// four copies of the table leave less of L1 to the voxel gathers; 5e5 photons
+// with null scores 963, 969 and 979 us. Few photons: 256, to reach more SMs.
+// GADJ_RESERVE bytes beside the table and the cells decide what is refused;
+// 128 threads' queues are less, so what it admits fits.
+constexpr size_t GADJ_RESERVE = 16 + 8 * (sizeof(double) + 384 * sizeof(float));
+static_assert(16 + 4 * (sizeof(double) + sizeof(float) * GADJ_QUEUE) <= GADJ_RESERVE, "what fits must fit 128 threads");
 cudaError_t grid_adjoint_block(const GridAdjArgs &a, int *block)
 {
     int dev = 0, sms = 0, optin = 0, per_sm = 0;
@@ -2410,9 +2439,11 @@ cudaError_t grid_adjoint_block(const GridAdjArgs &a, int *block)
     if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess) return e;
     const bool few = (a.g.m.n_photons + 31) / 32 < (unsigned long long)sms * (512 / 32);
-    const int order[3] = {few ? 256 : 512, few ? 512 : 1024, few ? 1024 : 256};
+    const int order[4] = {few ? 256 : 512, few ? 512 : 1024, few ? 1024 : 256, 128};
     int best = 0;
     *block = 0;
+    const size_t tb = a.g.c.phase_kind != MC_PHASE_HG ? a.g.c.table_bytes : 0;
+    if (tb + a.g.c.extra_bytes + GADJ_RESERVE > (size_t)optin) return cudaErrorInvalidValue;
     for (int b : order) {
         const size_t smem = grid_adjoint_smem(a, b);
         if (smem > (size_t)optin) continue;
@@ -2568,7 +2599,7 @@ int grid_adjoint_max_grid()
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    return sms * (2048 / GADJ_MIN_BLOCK);
+    return sms * 8;   // 1024 threads at the kernel's registers: 8 CTAs of the smallest size
 }
 
 cudaError_t launch_grid_adjoint(const GridAdjArgs &a, int rows, double *value, cudaStream_t st)

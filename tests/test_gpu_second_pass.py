@@ -33,7 +33,7 @@ def test_voxel_sums_match_the_homogeneous_gradient(gpu, ps_table, mu_a, kw):
     assert float(rho) * float(grad.double().sum()) == pytest.approx(mu_s * h[1] + mu_p * h[2], rel=2e-3)
 
 
-@pytest.mark.parametrize("n_bins,cell", [(64, 4), (8192, 4), (16384, 4), (8192, 1)])
+@pytest.mark.parametrize("n_bins,cell", [(64, 4), (8192, 4), (16384, 4), (8192, 1), (16384, 1)])
 @pytest.mark.parametrize("n", [50, 3_000, 100_000])
 def test_every_cta_size(gpu, n_bins, cell, n):
     """Few photons and large tables or many cells take other CTA sizes of the
