@@ -937,13 +937,16 @@ __global__ void __launch_bounds__(1024) walk_kernel(const __grid_constant__ Walk
     Smem S = carve<PHASE, SMEM_IMAGE>(smem, A.c);
     zero_tallies(S, A.c);
     if (threadIdx.x == 0) mbar_init(S.bar);
+    bool ready = true;
     if (PHASE != MC_PHASE_HG) {
-        if (!stage_bulk(S.table, A.m.table, A.c.table_bytes, S.bar, 0u, A.c.error)) return;
-        if (!bind_table<PHASE>(S, A.c)) return;
+        ready = stage_bulk(S.table, A.m.table, A.c.table_bytes, S.bar, 0u, A.c.error) && bind_table<PHASE>(S, A.c);
     } else {
         __syncthreads();
     }
-    wait_for_previous();   // the tallies and the counter are cleared
+    // the tallies and the counter are cleared; a CTA that leaves here waits as
+    // well, so that the end of this kernel always implies the end of the clearing
+    wait_for_previous();
+    if (!ready) return;
     Tally T;
     const LaunchRange R{A.counter, (uint32_t)A.m.n_photons};
     walk_loop<PHASE, SMEM_IMAGE, TRACE, UNIT>(A.c, A.m, A.m.rk, S, R, launch_pool(R), T);
@@ -1387,13 +1390,14 @@ __global__ void __launch_bounds__(1024) grid_kernel(const __grid_constant__ Grid
     const uint32_t tb = (PHASE != MC_PHASE_HG) ? A.c.table_bytes : 0u;
     float *s_maj = reinterpret_cast<float *>(smem + tb);
     uint32_t parity = 0u;
+    bool ready = true;
     if (PHASE != MC_PHASE_HG) {
-        if (!stage_bulk(S.table, A.m.table, A.c.table_bytes, S.bar, parity, A.c.error)) return;
+        ready = stage_bulk(S.table, A.m.table, A.c.table_bytes, S.bar, parity, A.c.error) && bind_table<PHASE>(S, A.c);
         parity ^= 1u;
-        if (!bind_table<PHASE>(S, A.c)) return;
     }
-    if (!stage_bulk(s_maj, A.maj, A.c.extra_bytes, S.bar, parity, A.c.error)) return;
-    wait_for_previous();   // the tallies and the counter are cleared
+    ready = ready && stage_bulk(s_maj, A.maj, A.c.extra_bytes, S.bar, parity, A.c.error);
+    wait_for_previous();   // as in walk_kernel
+    if (!ready) return;
     Tally T;
     grid_loop<PHASE, SMEM_IMAGE, TRACE, UNIT>(A, S, s_maj, T);
     flush<SMEM_IMAGE>(A.c, A.m, S, T);
