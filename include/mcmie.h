@@ -290,12 +290,12 @@ mc_status mc_run_static(const mc_medium *medium, const mc_geometry *geom,
 
 /* Many media in one launch: the CTAs are shared out among the media by
  * estimated photon-steps; a CTA's warps take chunks of at most item_photons
- * photons (0: 128; else 32 .. 2^20; fewer as the medium's photons run out)
- * of its medium from that medium's counter, and
- * when the medium's photons are all taken the CTA flushes its tallies into
- * the medium's, joins the medium with most work left per CTA (staging its
- * table in shared memory) and goes on, so the media follow one
- * another without launch gaps. All instances share geometry, camera and run
+ * photons (0: 128; else 32 .. 2^20, of which 2^15 are used at most; fewer as
+ * the medium's photons run out) of its medium from that medium's counter, and
+ * when the medium's photons are all taken the CTA flushes its tallies into the
+ * medium's, joins the medium with most work left per CTA (staging its table in
+ * shared memory) and goes on, so the media follow one another without launch
+ * gaps. All instances share geometry, camera and run
  * parameters (run->n_photons, photon_offset and seed are ignored; each
  * instance has its own), and one phase kind and table size. Tallies per
  * instance as for mc_run, bit-identical to running each instance with

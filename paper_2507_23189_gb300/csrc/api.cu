@@ -12,6 +12,7 @@
 #include <new>
 
 #include "engine.h"
+#include "tally.h"
 #include "table_format.h"
 
 namespace {
@@ -172,7 +173,8 @@ void fill_common(mcx::CommonArgs &c, const mc_medium *m, const mc_geometry *g, c
     c.inv_rr_surv = r->rr_survival > 0 ? (float)(1.0 / r->rr_survival) : 0.0f;
     c.max_events = r->max_events;
     c.scatter_cap = r->max_scatter ? r->max_scatter : 0xFFFFFFFFu;
-    c.ev_stop = std::min(c.max_events, c.scatter_cap);
+    c.ev_look = std::min(c.max_events, mcx::LOOK_FLIGHTS);
+    c.ev_stop = std::min(c.ev_look, c.scatter_cap);
     c.img_scale = std::ldexp(1.0f, frac_bits_of(r, n_photons));
     c.error = error;
     c.extra_bytes = 0;
@@ -391,7 +393,7 @@ mc_status mc_run_batch(int n, const mc_instance *inst, const mc_geometry *geom, 
     for (int i = 0; i < n; ++i) n_max = inst[i].n_photons > n_max ? inst[i].n_photons : n_max;
     fill_common(a->c, &inst[0].medium, geom, camera, run, d_error, n_max);
     a->n_media = n;
-    a->max_per = item_photons ? (unsigned)(item_photons / 32) : 4u;
+    a->max_per = item_photons ? std::min((unsigned)item_photons, mcx::MAX_ITEM) / 32 : 4u;
     a->counters = static_cast<unsigned long long *>(d_work);
     double total = 0.0, sum = 0.0;
     for (int i = 0; i < n; ++i) {

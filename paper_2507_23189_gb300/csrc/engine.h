@@ -43,7 +43,8 @@ struct CommonArgs {
     float rr_thr, rr_surv, inv_rr_surv;
     uint32_t max_events;
     uint32_t scatter_cap;       // collisions a photon may have (max_scatter, or 2^32 - 1 for none)
-    uint32_t ev_stop;           // min(max_events, scatter_cap)
+    uint32_t ev_look;           // min(max_events, LOOK_FLIGHTS of the flight counts)
+    uint32_t ev_stop;           // min(ev_look, scatter_cap)
     float img_scale;            // 2^image_frac_bits
     uint32_t *error;
     // image rows [band0, band0 + band_rows) are privatised in shared memory

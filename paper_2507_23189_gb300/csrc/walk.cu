@@ -21,6 +21,7 @@
 
 #include "engine.h"
 #include "table_format.h"
+#include "tally.h"
 
 namespace mcx {
 namespace {
@@ -583,12 +584,14 @@ __device__ __forceinline__ bool bind_table(Smem &S, const CommonArgs &C)
     return true;
 }
 
-// Per-thread tallies, reduced when a CTA finishes a medium.
-struct Tally {
-    uint32_t steps = 0;         // flushed per medium; a thread's counts per flush fit 32 bits
-    uint32_t n_refl = 0, n_far = 0, n_side = 0, n_ball = 0;   // photons of weight one
-    long long refl = 0, far = 0, side = 0, ball = 0, abs = 0; // 2^-32 weight units
-};
+// The thread's flights, handed on when they are due (see Tally): straight into
+// global memory, one instruction where the CTA's total in shared memory takes a
+// dozen (1 % of the walk at tau 5, for all that it is hardly ever reached).
+__device__ __forceinline__ void hand_on(const MediumArgs &M, Tally &T)
+{
+    const uint32_t n = T.due();
+    if (n) atomicAdd(&M.totals[MC_TOT_STEPS], (unsigned long long)n);
+}
 
 // Warp -> shared -> the medium's global tallies (one atomic per nonzero entry).
 template <bool SMEM_IMAGE>
@@ -692,9 +695,10 @@ struct Pool {                                // all warp-uniform
     bool dry = false;                        // the range is used up
 
     // The next photon of each lane in `need` (the limit or beyond: none). The
-    // whole warp calls it.
-    template <class Range>
-    __device__ __forceinline__ uint32_t take(const Range &R, unsigned need)
+    // whole warp calls it. more(): called by all lanes before more photons are
+    // taken from the range.
+    template <class Range, class More>
+    __device__ __forceinline__ uint32_t take(const Range &R, unsigned need, More more)
     {
         const int lane = threadIdx.x & 31;
         const uint32_t n = __popc(need), rank = __popc(need & ((1u << lane) - 1u)), avail = end - next;
@@ -705,6 +709,7 @@ struct Pool {                                // all warp-uniform
         uint32_t base = R.limit;
         const uint32_t first = next;
         if (!dry) {
+            more();
             const uint32_t take = 32u * R.per(seen);
             unsigned long long b = 0;
             if (lane == 0) b = min(R.grab(take), (unsigned long long)R.limit);
@@ -778,7 +783,7 @@ __device__ __forceinline__ void walk_loop(const CommonArgs &C, const MediumArgs 
     while (true) {
         const unsigned need = __ballot_sync(FULL, !alive);
         if (need) {
-            const uint32_t mine = P.take(R, need);
+            const uint32_t mine = P.take(R, need, [&] { hand_on(M, T); });
             if (!alive && mine < R.limit) start(mine);
             if (P.dry && !__any_sync(FULL, alive)) break;
         }
@@ -868,6 +873,7 @@ __device__ __forceinline__ void walk_loop(const CommonArgs &C, const MediumArgs 
 
         if (TRACE) {
             int status = 0;
+            if (ev >= LOOK_FLIGHTS) hand_on(M, T);
             if (ev >= C.scatter_cap) {
                 sadd64(&s_tot[MC_TOT_TRUNC], fix32(w));
                 status = 5;
@@ -902,6 +908,7 @@ __device__ __forceinline__ void walk_loop(const CommonArgs &C, const MediumArgs 
             // max_scatter ends here and never uses it)
             scatter<PHASE>(M, C, S, rnd.y, u2, dx, dy, dz);
             if ((ev >= C.ev_stop) | (!UNIT && ((w < C.rr_thr) | !(w == w)))) {
+                if (ev >= LOOK_FLIGHTS) hand_on(M, T);
                 if (ev >= C.scatter_cap) {
                     sadd64(&s_tot[MC_TOT_TRUNC], fix32(w));
                     alive = false;
@@ -1247,18 +1254,21 @@ __device__ __forceinline__ void grid_loop(const GridArgs &G, const Smem &S, cons
     while (true) {
         const unsigned need = __ballot_sync(FULL, !alive);
         if (need) {
-            const uint32_t mine = P.take(R, need);
+            const uint32_t mine = P.take(R, need, [&] { hand_on(M, T); });
             if (!alive && mine < R.limit) start(mine);
             if (P.dry && !__any_sync(FULL, alive)) break;
         }
         if (!alive) continue;
 
-        if (ev >= C.max_events) {
-            sadd64(&s_tot[MC_TOT_TRUNC], fix32(w));
-            atomicOr(C.error, MC_EFLAG_EVENTS);
-            trace_write<TRACE>(C, rel, ncoll, 6, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, -1, -1, -1);
-            alive = false;
-            continue;
+        if (ev >= C.ev_look) {
+            hand_on(M, T);
+            if (ev >= C.max_events) {
+                sadd64(&s_tot[MC_TOT_TRUNC], fix32(w));
+                atomicOr(C.error, MC_EFLAG_EVENTS);
+                trace_write<TRACE>(C, rel, ncoll, 6, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, -1, -1, -1);
+                alive = false;
+                continue;
+            }
         }
         const uint4 rnd = philox10(make_uint4(pk0, pk1, ev, 0u), M.rk);
         ++ev;
@@ -1685,7 +1695,7 @@ __global__ void __launch_bounds__(GADJ_MAX_BLOCK) grid_adjoint_kernel(const __gr
     while (true) {
         const unsigned need = __ballot_sync(FULL, !alive);
         if (need) {
-            const uint32_t mine = pool.take(R, need);
+            const uint32_t mine = pool.take(R, need, [] {});
             if (!alive && mine < R.limit) start(mine);
             if (!__any_sync(FULL, alive)) break;
         }
@@ -2031,7 +2041,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
     while (true) {
         const unsigned need = __ballot_sync(FULL, !alive);
         if (need) {
-            const uint32_t mine = pool.take(R, need);
+            const uint32_t mine = pool.take(R, need, [] {});
             if (!alive && mine < R.limit) start(mine);
             if (!__any_sync(FULL, alive)) break;
         }
