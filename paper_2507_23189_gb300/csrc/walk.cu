@@ -1028,7 +1028,12 @@ __global__ void __launch_bounds__(1024) batch_kernel(const __grid_constant__ Bat
             }
         }
         __syncthreads();
-        const int m = (int)(long long)S.item[0];
+        // the same for every thread, which the compiler sees from the shuffle
+        // alone: with the medium's arguments and round keys in uniform registers
+        // the H-G forms take 44 to 48 registers, else 64 and up to 160 bytes of
+        // spills (64 media of 2e5 photons 429 -> 409 us, of 1e7 17.05 -> 16.25
+        // ms, absorbing 19.13 -> 17.55 ms; the table forms do it either way)
+        const int m = __shfl_sync(FULL, (int)(long long)S.item[0], 0);
         const unsigned long long joined = S.item[1];
         __syncthreads();
         if (m < 0) break;
