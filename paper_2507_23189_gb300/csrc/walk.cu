@@ -1019,7 +1019,8 @@ __global__ void __launch_bounds__(1024) batch_kernel(const __grid_constant__ Bat
                 while (m < B.n_media - 1 && B.share[m] <= mine) ++m;
                 const unsigned long long next =
                     *reinterpret_cast<volatile unsigned long long *>(B.counters + m) & (JOIN - 1);
-                if (next >= B.m[m].n_photons) m = -1;
+                // one lane's reading: the counter moves, and the warp goes on together
+                m = __shfl_sync(FULL, next >= B.m[m].n_photons ? -1 : m, 0);
             }
             if (m < 0) m = pick_medium(B, threadIdx.x);
             if (threadIdx.x == 0) {
