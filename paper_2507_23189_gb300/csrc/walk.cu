@@ -20,6 +20,7 @@
 #include <stdint.h>
 
 #include "engine.h"
+#include "sums.h"
 #include "table_format.h"
 #include "tally.h"
 
@@ -2188,16 +2189,17 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
         row[threadIdx.x] = t;
     }
     if (PHASEW) {
-        // hat k's private sums: a compensated single-precision sum, each thread
-        // starting at another column so that a warp's lanes read different
-        // banks. (Double sums over one bank kept the double-precision pipe
-        // busy for 26 of the kernel's 152 us at 1e6 photons and 64 hats.)
+        // hat k's private sums, each thread starting at another column so that a
+        // warp's lanes read different banks, on the single-precision pipe (double
+        // sums over one bank kept the double-precision pipe busy for 26 of the
+        // kernel's 152 us at 1e6 photons and 64 hats; a Kahan pair would save 2 us
+        // more and be off by up to 32 times as much)
         double gzb = 0.0;
         for (int q = 0; q < warps; ++q) gzb += s_red[q * 4 + 3];
         for (int k = threadIdx.x; k < nw; k += B) {
-            float sum = 0.f, comp = 0.f;
-            for (int q = 0; q < B; ++q) kahan_add(sum, comp, rows[k * B + ((q + k) & (B - 1))]);
-            row[3 + k] = ((double)sum - (double)comp) - s_z[k] * gzb;
+            Sum3 sum;
+            for (int q = 0; q < B; ++q) sum.add(rows[k * B + ((q + k) & (B - 1))]);
+            row[3 + k] = sum.value() - s_z[k] * gzb;
         }
     }
 }
