@@ -104,24 +104,28 @@ __device__ __forceinline__ float mc_log(float x)   // x normal
     return y * 0.693147180559945309417f;
 #endif
 }
-__device__ __forceinline__ float mc_exp(float x)    // results below 2^-126 become 0
-{
-#ifdef MC_STRICT
-    return expf(x);
-#else
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x * 1.44269504088896340736f));
-    return y;
-#endif
-}
-__device__ __forceinline__ float mc_exp2(float x)   // results below 2^-126 become 0
+// TALLY: results below 2^-126 become 0, far below half a unit of any image
+// tally. Traces and gradients have no such unit and keep them (0.8 % of the
+// gradient of mu_s and mu_a, 0.5 % of a null-score step).
+template <bool TALLY>
+__device__ __forceinline__ float mc_exp2(float x)
 {
 #ifdef MC_STRICT
     return exp2f(x);
 #else
     float y;   // the hardware approximation, relative error a few 1e-7
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    if (TALLY) asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    else asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+#endif
+}
+template <bool TALLY>
+__device__ __forceinline__ float mc_exp(float x)
+{
+#ifdef MC_STRICT
+    return expf(x);
+#else
+    return mc_exp2<TALLY>(x * 1.44269504088896340736f);
 #endif
 }
 __device__ __forceinline__ void mc_sincos(float x, float *s, float *c)
@@ -867,7 +871,7 @@ __device__ __forceinline__ void walk_loop(const CommonArgs &C, const MediumArgs 
         // camera: next-event estimate toward +y
         int nb, ix, iz;
         const float psr = camera_psr<PHASE>(M, C, S, dy, nb);
-        const float nee = w * psr * mc_exp2(fmaf(cam_a, ry, cam_b));
+        const float nee = w * psr * mc_exp2<!TRACE>(fmaf(cam_a, ry, cam_b));
         const int pix = camera_pixel_inside(C, rx, rz, ix, iz);   // 0 < rx < lx, |rz| < hz tested above
         const float vf = nee * C.img_scale;
         image_add<SMEM_IMAGE>(s_img, C, M.image, pix, vf);
@@ -1342,7 +1346,7 @@ __device__ __forceinline__ void grid_loop(const GridArgs &G, const Smem &S, cons
         int nb, pix_x, pix_z;
         const float psr = camera_psr<PHASE>(M, C, S, dy, nb);
         const float top = (iy == G.gy - 1) ? C.hy : fmaf((float)(iy + 1), G.vy, -C.hy);
-        const float nee = w * psr * mc_exp(-fmaf(cell.x, top - ry, cell.y));
+        const float nee = w * psr * mc_exp<!TRACE>(-fmaf(cell.x, top - ry, cell.y));
         const int pix = camera_pixel(C, rx, rz, pix_x, pix_z);
         const float vf = nee * C.img_scale;
         image_add<SMEM_IMAGE>(s_img, C, M.image, pix, vf);
@@ -1765,7 +1769,7 @@ __global__ void __launch_bounds__(GADJ_MAX_BLOCK) grid_adjoint_kernel(const __gr
                     int nb, pix_x, pix_z;
                     const float psr = camera_psr<PHASE>(M, C, S, dy, nb);
                     const float top = (iy == G.gy - 1) ? C.hy : fmaf((float)(iy + 1), G.vy, -C.hy);
-                    const float nee = w * psr * mc_exp(-fmaf(cell.x, top - ry, cell.y));
+                    const float nee = w * psr * mc_exp<false>(-fmaf(cell.x, top - ry, cell.y));
                     const int pix = camera_pixel(C, rx, rz, pix_x, pix_z);
                     const float Aj = __ldg(&A.adj[pix]) * nee;
                     if (total != 0) {
@@ -2088,7 +2092,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
             int nb, ix, iz;
             const float psr = camera_psr<PHASE>(M, C, S, dy, nb);
             const float l = C.hy - ry;
-            const float nee = w * psr * mc_exp(-M.mu_ext * l);
+            const float nee = w * psr * mc_exp<false>(-M.mu_ext * l);
             const int pix = camera_pixel(C, rx, rz, ix, iz);
             const float Aj = __ldg(&A.adj[pix]) * nee;
             P += Aj;
