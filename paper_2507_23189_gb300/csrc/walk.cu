@@ -1458,15 +1458,21 @@ constexpr int QEX = 6 * GADJ_COLS, QCOEF = 7 * GADJ_COLS, QEY = 8 * GADJ_COLS, Q
               QPOINT = 10 * GADJ_COLS, QCOLUMN = 11 * GADJ_COLS;
 constexpr int QLEN = QEX;         // while it is rasterised: the length, negative inside the box around the beam axis
 
-// float -> double by moving the bit fields, on the integer pipe (GB300's
-// double-precision pipe, which converts, takes 2 lanes per clock and SM):
-// exact for normal numbers, infinities and NaN; zero and subnormals come out
-// below 2^-126, far under any term summed here.
-__device__ __forceinline__ double widen(float f)
+// f as a double by moving the bit fields, on the integer pipe (GB300's
+// double-precision pipe, which converts, takes 2 lanes per clock and SM): exact
+// for normal numbers, infinities and NaN; not for zero and subnormals. bias:
+// 896 less the power of two to divide by, in the exponent's place.
+__device__ __forceinline__ double widen(float f, int bias = 0x38000000)
 {
-    const int hi = (int)(((uint32_t)(__float_as_int(f) >> 3) & 0x8FFFFFFFu) + 0x38000000u);   // exponent + 896
+    const int hi = (int)(((uint32_t)(__float_as_int(f) >> 3) & 0x8FFFFFFFu) + bias);   // exponent + 896
     const int lo = (int)(__float_as_uint(f) << 29);
     return __hiloint2double(fabsf(f) < __int_as_float(0x7f800000) ? hi : hi | 0x7FF00000, lo);
+}
+// *slot() += f; zero and subnormals are not added (slot is not called).
+template <class Slot>
+__device__ __forceinline__ void add_wide(float f, Slot slot)
+{
+    if (!(fabsf(f) < 1.17549435e-38f)) atomicAdd(slot(), widen(f));
 }
 
 __device__ __forceinline__ float rcp_approx(float x)
@@ -1508,7 +1514,10 @@ __device__ __forceinline__ void raster_unit(const GridAdjArgs &A, double *bgs, c
 {
     const GridArgs &G = A.g;
     const float *f = s_seg + q;
-    const float coef = f[QCOEF];
+    // a small coefficient times 2^64, for pieces that are normal numbers
+    const bool small = fabsf(f[QCOEF]) < 2.32830644e-10f;
+    const float coef = small ? f[QCOEF] * 18446744073709551616.f : f[QCOEF];
+    const int bias = small ? 0x38000000 - (64 << 20) : 0x38000000;
     const bool last = u == units - 1, box = f[QLEN] < 0.f;
     double *grad = box ? bgs : A.gsum;
     const int span = box ? (int)A.nbox : G.gx * G.gy * G.gz;
@@ -1547,7 +1556,7 @@ __device__ __forceinline__ void raster_unit(const GridAdjArgs &A, double *bgs, c
     for (int it = 0; it < 3 * 4096; ++it) {
         const float m = fminf(fminf(next[0], next[1]), next[2]);
         if (!(m <= t1)) break;
-        if (m > t) atomicAdd(&grad[chk(v, span, G.c.error)], widen(coef * (m - t)));
+        if (m > t) atomicAdd(&grad[chk(v, span, G.c.error)], widen(coef * (m - t), bias));
         t = m;
 #pragma unroll
         for (int a = 0; a < 3; ++a)
@@ -1557,7 +1566,7 @@ __device__ __forceinline__ void raster_unit(const GridAdjArgs &A, double *bgs, c
                 next[a] = fmaxf(fmaf(j[a], dl[a], first[a]), 0.f);
             }
     }
-    if (last && t1 > t) atomicAdd(&grad[chk(v, span, G.c.error)], widen(coef * (t1 - t)));
+    if (last && t1 > t) atomicAdd(&grad[chk(v, span, G.c.error)], widen(coef * (t1 - t), bias));
 }
 
 // The voxel's element in the sums: inside the box around the beam axis, in this
@@ -1593,8 +1602,8 @@ __device__ __forceinline__ void raster_queue(const GridAdjArgs &A, double *bgs, 
             const int iz = centred_cell(rz, G.inv_vz, 0.5f * (float)G.gz, G.gz);
             const size_t v = chk((iz * G.gy + iy) * G.gx + ix, G.gx * G.gy * G.gz, G.c.error);
             const float gv = f[QPOINT], Aj = f[QCOLUMN];
-            if (gv != 0.f) atomicAdd(box_slot(A, A.gsum, bgs, ix, iy, iz, v), widen(gv));
-            if (Aj != 0.f) atomicAdd(box_slot(A, A.s1, bs1, ix, iy, iz, v), widen(Aj));
+            add_wide(gv, [&] { return box_slot(A, A.gsum, bgs, ix, iy, iz, v); });
+            add_wide(Aj, [&] { return box_slot(A, A.s1, bs1, ix, iy, iz, v); });
             const float ex = rx - px, ey = ry - py, ez = rz - pz;
             const float len = sqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez)));
             // inside the box by a voxel at both ends (it is convex)?
@@ -1759,7 +1768,8 @@ __global__ void __launch_bounds__(GADJ_MAX_BLOCK) grid_adjoint_kernel(const __gr
                 if (NULLS && !(u3 < acc) && total != 0) {
                     // null collision: its score times the camera terms after it
                     const float B = Ptot - P;
-                    if (B != 0.f) atomicAdd(box_slot(A, gs, bgs, ix, iy, iz, v), widen(-B * mc_div_n(A.k_ext, mb - cell.x)));
+                    if (B != 0.f)
+                        add_wide(-B * mc_div_n(A.k_ext, mb - cell.x), [&] { return box_slot(A, gs, bgs, ix, iy, iz, v); });
                 }
                 if (u3 < acc) {
                     u3 = mc_div_n(u3, acc);
@@ -1790,7 +1800,7 @@ __global__ void __launch_bounds__(GADJ_MAX_BLOCK) grid_adjoint_kernel(const __gr
                                 double *ex = iy == G.gy / 2 && iz == G.gz / 2
                                                  ? A.exr + (size_t)(blockIdx.x % (unsigned)kRowCopies) * G.gx + ix
                                                  : A.ex + v;
-                                atomicAdd(ex, widen(coef));
+                                add_wide(coef, [&] { return ex; });
                             } else {
                                 float *q = s_seg + atomicAdd(s_cnt, 1);
                                 q[0] = px; q[GADJ_COLS] = py; q[2 * GADJ_COLS] = pz;
@@ -1801,8 +1811,8 @@ __global__ void __launch_bounds__(GADJ_MAX_BLOCK) grid_adjoint_kernel(const __gr
                             }
                         }
                         if (!queued) {
-                            if (gv != 0.f) atomicAdd(box_slot(A, gs, bgs, ix, iy, iz, v), widen(gv));
-                            if (Aj != 0.f) atomicAdd(box_slot(A, s1c, bs1, ix, iy, iz, v), widen(Aj));
+                            add_wide(gv, [&] { return box_slot(A, gs, bgs, ix, iy, iz, v); });
+                            add_wide(Aj, [&] { return box_slot(A, s1c, bs1, ix, iy, iz, v); });
                         }
                     }
                     P += Aj;

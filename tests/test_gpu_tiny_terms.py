@@ -1,11 +1,38 @@
-"""Gradient terms at the bottom of the single-precision range: camera
-transmittances below 2^-126 still count in the gradients of the coefficients."""
+"""Gradient terms at the bottom of the single-precision range: those of a density
+gradient add nothing beyond their own size, and camera transmittances below
+2^-126 still count in the gradients of the coefficients."""
 import math
 
 import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("nulls", [None, 1.5])
+@pytest.mark.parametrize("power", [-100, -130, -145])
+def test_terms_below_the_normal_range(gpu, ps_table, nulls, power):
+    import torch
+    geo = gpu.Geometry(45.0, 10.0, 10.0)
+    e = gpu.Engine(gpu.Camera(16, 16, 8), geo)
+    grid = gpu.Grid(torch.full((12, 40, 16), 0.2, device="cuda"), 1.0, 1.0, 0.0, (4, 8, 4)).prepare(geo)
+    med = gpu.Medium(1.0, 0.0, "table", 0.0, ps_table)
+
+    def gradient(adj):
+        _, grad = e.grid_adjoint(grid, med, torch.full((16, 16), adj), 20_000, seed=2, nulls=nulls)
+        e.check()
+        return grad.double().cpu().numpy()
+
+    one, small = gradient(1.0), gradient(2.0 ** power)
+    size = np.abs(one).sum() * 2.0 ** power
+    if power == -100:
+        # the same photons; a term comes from a product of four numbers at most,
+        # of which 2^-100 takes none out of the normal range but the smallest
+        np.testing.assert_allclose(small * 2.0 ** 100, one, rtol=1e-4, atol=1e-6 * np.abs(one).max())
+    # terms that are too small are dropped or rounded to multiples of 2^-149:
+    # an entry is then off by its terms' own size at most, which cancellation
+    # may leave 2^10 times the entries', plus half a unit
+    assert np.abs(small).sum() <= 2.0 ** 10 * size + one.size * 2.0 ** -149
 
 
 @pytest.mark.parametrize("n_w", [0, 8])
