@@ -189,8 +189,8 @@ __global__ void __launch_bounds__(COL_BLOCK) fold_kernel(const double *__restric
                                                          int gx, int gy, int gz, double k_vy)
 {
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const unsigned lanes = __ballot_sync(FULL, t < (long long)gx * gz);   // those with a column
     if (t >= (long long)gx * gz) return;
-    const unsigned lanes = __activemask();
     const int iz = (int)(t / gx), ix = (int)(t - (long long)iz * gx);
     const size_t base = (size_t)iz * gy * gx + ix;
     double run = 0.0;
