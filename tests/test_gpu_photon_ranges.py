@@ -58,4 +58,8 @@ def test_grid_and_adjoint_ranges(gpu, ps_table, n):
         value, _ = e.grid_adjoint(grid, med, adj, n, seed=9, nulls=nulls)
         if nulls is None:       # scaled majorants draw other paths
             assert abs(float(value) - want) <= 1e-5 * abs(want) + n * 20 * 2.0 ** -32
+        cut = n // 3            # the same photons in two calls; their terms are
+        parts = [float(e.grid_adjoint(grid, med, adj, m, seed=9, nulls=nulls, photon_offset=o)[0])
+                 for m, o in ((cut, 0), (n - cut, cut))]       # summed in double
+        assert abs(float(value) - sum(parts)) <= n * 2.0 ** -53 * abs(float(value))
     e.check()

@@ -1,7 +1,8 @@
 """The variant for media that never change a photon's weight against the
 general one. A weight threshold of 1 keeps the variant; a threshold of 2 with
 certain survival takes the general walk, whose roulette then multiplies by 1:
-the same photons, so the same integers. Absorption, however small, counts."""
+the same photons, so the same integers. Absorption that leaves an albedo below
+1 in single precision counts."""
 import numpy as np
 import pytest
 
@@ -77,3 +78,25 @@ def test_adjoint(gpu, ps_table, phase, n_w):
     # the same terms in single precision, added in another order: compensated
     # sums, and private sums of a few terms each over the hats
     np.testing.assert_allclose(got[0], got[1], rtol=2e-6, atol=2e-6 * np.abs(got[1]).max())
+
+
+def test_albedos_next_to_one(gpu, ps_table):
+    """The largest single below 1 captures 2^-24 of the weight at each collision;
+    an albedo that rounds to 1 captures nothing in either variant."""
+    e = gpu.Engine(gpu.Camera(16, 16, 8), gpu.Geometry(45.0, 10.0, 10.0))
+    n, mu = 20_000, 0.25
+
+    def run(phase, absorbed, **rr):
+        e.run(gpu.Medium(mu * (1.0 - absorbed), mu * absorbed, phase, 0.87, ps_table), n, seed=1, **rr)
+        return _state(e)
+
+    for phase in ("table", "hg"):
+        totals = run(phase, 2.0 ** -24)[2]
+        collisions = int(totals[7]) - n               # flights less exits: no photon is truncated
+        # 2^-24 is 256 units of 2^-32; a photon's later captures are of a weight
+        # that single precision holds to within 2^-24
+        assert collisions > n and abs(int(totals[3]) - 256 * collisions) <= collisions
+        unit, general = run(phase, 2.0 ** -26, **UNIT), run(phase, 2.0 ** -26, **GENERAL)
+        assert int(unit[2][3]) == 0
+        for a, b in zip(unit, general):
+            np.testing.assert_array_equal(a, b)
