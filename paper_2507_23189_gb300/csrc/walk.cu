@@ -2360,9 +2360,8 @@ cudaError_t launch_persistent(Kern kern, const void *args_unused, const LaunchCf
     return cudaSuccess;
 }
 
-// Where the image accumulates and how big the CTA is for a launch over n_photons.
-// Sets c.band0/band_rows.
-cudaError_t plan_image(CommonArgs &c, LaunchCfg &cfg, unsigned long long n_photons, bool *smem_img, size_t *smem)
+// Where the image accumulates and how big the CTA is. Sets c.band0/band_rows.
+cudaError_t plan_image(CommonArgs &c, LaunchCfg &cfg, bool *smem_img, size_t *smem)
 {
     const size_t tb = ((c.phase_kind != MC_PHASE_HG) ? c.table_bytes : 0) + c.extra_bytes;
     const size_t tail = sizeof(unsigned long long) * (c.n_radial + MC_N_TOTALS + 3) + 16;
@@ -2403,17 +2402,12 @@ cudaError_t plan_image(CommonArgs &c, LaunchCfg &cfg, unsigned long long n_photo
         if (b0 > c.nz - c.band_rows) b0 = c.nz - c.band_rows;
         c.band0 = b0 < 0 ? 0 : b0;
     }
-    // fewer photons than lanes on the chip: CTAs of as few warps (8 at least, for
-    // the tallies' clearing and flushing) as spread them over all SMs
     c.band_first = c.band0 * c.nx;
     c.band_pixels = c.band_rows * c.nx;
-    if (cfg.block == 0) {
-        int sms = 0;
-        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        const unsigned long long warps = (n_photons + 31) / 32;
-        const unsigned long long per_sm_warps = (warps + sms - 1) / sms;
-        cfg.block = mode != 3 || per_sm_warps <= 8 ? 256 : (per_sm_warps >= 32 ? 1024 : 32 * (int)per_sm_warps);
-    }
+    // also for few photons: warps without any still clear and flush the CTA's
+    // part of the image (20 000 photons on 512 x 512 pixels: 25 us a call, 35
+    // with CTAs of 256 threads)
+    if (cfg.block == 0) cfg.block = mode == 3 ? 1024 : 256;
     *smem = tb + tail + (*smem_img ? row * c.band_rows : 0);
     if (*smem > (size_t)optin) return cudaErrorInvalidValue;
     return cudaSuccess;
@@ -2566,7 +2560,7 @@ cudaError_t launch_walk(const WalkArgs &a0, bool fresh, bool trace, const Launch
     LaunchCfg cfg = cfg0;
     bool smem_img = false;
     size_t smem = 0;
-    cudaError_t e = plan_image(a.c, cfg, a.m.n_photons, &smem_img, &smem);
+    cudaError_t e = plan_image(a.c, cfg, &smem_img, &smem);
     if (e != cudaSuccess) return e;
     if ((e = launch_zero(a, fresh, st)) != cudaSuccess || a.m.n_photons == 0) return e;
     if ((e = launch_walk_kernel(a, trace, cfg, smem_img, smem, st)) != cudaSuccess) return e;
@@ -2579,7 +2573,7 @@ cudaError_t check_plan(const CommonArgs &c0, const LaunchCfg &cfg0)
     LaunchCfg cfg = cfg0;
     bool smem_img = false;
     size_t smem = 0;
-    return plan_image(c, cfg, 0, &smem_img, &smem);
+    return plan_image(c, cfg, &smem_img, &smem);
 }
 
 namespace {
@@ -2618,7 +2612,7 @@ cudaError_t launch_grid(const GridArgs &a0, bool fresh, bool trace, const Launch
     LaunchCfg cfg = cfg0;
     bool smem_img = false;
     size_t smem = 0;
-    cudaError_t e = plan_image(a.c, cfg, a.m.n_photons, &smem_img, &smem);
+    cudaError_t e = plan_image(a.c, cfg, &smem_img, &smem);
     if (e != cudaSuccess) return e;
     WalkArgs w;
     w.c = a.c;
@@ -2665,7 +2659,7 @@ cudaError_t launch_batch(const BatchArgs &a0, bool fresh, const LaunchCfg &cfg0,
     size_t smem = 0;
     unsigned long long photons = 0;
     for (int i = 0; i < a.n_media; ++i) photons += a.m[i].n_photons;
-    cudaError_t e = plan_image(a.c, cfg, photons, &smem_img, &smem);
+    cudaError_t e = plan_image(a.c, cfg, &smem_img, &smem);
     if (e != cudaSuccess) return e;
     batch_zero_kernel<<<dim3(fresh ? sign_blocks(a.c) : 1, (unsigned)a.n_media), ZERO_BLOCK, 0, st>>>(a, fresh);
     if ((e = cudaGetLastError()) != cudaSuccess || !photons) return e;
