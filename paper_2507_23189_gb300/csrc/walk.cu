@@ -652,6 +652,7 @@ __device__ void flush(const CommonArgs &C, const MediumArgs &M, const Smem &S, T
 // ends, but at 20 to 60 photons per lane that is up to 22 % slower: lanes end
 // their last shares alone.)
 constexpr uint32_t MAX_PER = 4;
+constexpr float GRAB_SHARE = 0.5f / 32.f;
 
 // A launch's range [0, limit): warps get their first 32 per photons by their
 // number (interleaved over the CTAs, so that a small range is spread over all
@@ -660,10 +661,11 @@ constexpr uint32_t MAX_PER = 4;
 struct LaunchRange {
     unsigned long long *counter;
     uint32_t limit;             // photons, at most 2^31
+    float share = GRAB_SHARE;   // of an even split of what is left, over the 32 lanes
     __device__ __forceinline__ uint32_t warps() const { return gridDim.x * (blockDim.x >> 5); }
     __device__ __forceinline__ uint32_t per(uint32_t seen) const
     {
-        return min(max((uint32_t)((float)(limit - seen) * (0.015625f / (float)warps())), 1u), MAX_PER);
+        return min(max((uint32_t)((float)(limit - seen) * (share / (float)warps())), 1u), MAX_PER);
     }
     __device__ __forceinline__ unsigned long long first(uint32_t warp) const
     {
@@ -962,7 +964,7 @@ __global__ void __launch_bounds__(1024) walk_kernel(const __grid_constant__ Walk
     wait_for_previous();
     if (!ready) return;
     Tally T;
-    const LaunchRange R{A.counter, (uint32_t)A.m.n_photons};
+    const LaunchRange R{A.counter, (uint32_t)A.m.n_photons, A.c.grab_share};
     walk_loop<PHASE, SMEM_IMAGE, TRACE, UNIT>(A.c, A.m, A.m.rk, S, R, launch_pool(R), T);
     flush<SMEM_IMAGE>(A.c, A.m, S, T);
 }
@@ -2409,6 +2411,12 @@ cudaError_t plan_image(CommonArgs &c, LaunchCfg &cfg, bool *smem_img, size_t *sm
     }
     c.band_first = c.band0 * c.nx;
     c.band_pixels = c.band_rows * c.nx;
+    // an image beyond L2 (129 MB): the counter's atomics queue behind the image's
+    // traffic to memory, and larger, fewer chunks end sooner (8192 x 4096 pixels,
+    // 3e5, 1e6 and 1e7 photons 233, 294 and 931 us a call with half an even
+    // share, 200, 262 and 905 with two; 2048 x 2048, 1e6: 80 against 86)
+    const bool beyond = sizeof(unsigned long long) * (size_t)c.nx * c.nz >= ((size_t)1 << 27);
+    c.grab_share = beyond ? 4.f * GRAB_SHARE : GRAB_SHARE;
     // also for few photons: warps without any still clear and flush the CTA's
     // part of the image (20 000 photons on 512 x 512 pixels: 25 us a call, 35
     // with CTAs of 256 threads)
