@@ -751,7 +751,10 @@ mc_status grid_adjoint_common(const mc_grid *g, const void *d_grid_work, const m
     // s1, gsum, the box copies of s1 and of gsum; exact: the row copies of ex,
     // then ex itself (not for a pencil beam, whose first flights lie in one row)
     const int bw = std::min(mcx::kBoxWidth, std::min(g->gy, g->gz));
-    const size_t bb = up(sizeof(double) * box_voxels(g)), cb = (size_t)mcx::kBoxCopies * bb;
+    // no more copies than CTAs (of 4 warps at least, all but the last with photons)
+    // can add to: one photon on 2048 x 32 x 32 voxels 226 us a call with 8
+    const int copies = (int)std::min<uint64_t>(mcx::kBoxCopies, (run->n_photons + 127) / 128);
+    const size_t bb = up(sizeof(double) * box_voxels(g)), cb = (size_t)copies * bb;
     const size_t rb = up(sizeof(double) * (size_t)mcx::kRowCopies * g->gx);
     const size_t main = 2 * nb, sums = main + 2 * cb + (nulls ? 0 : rb), region = sums + (nulls ? 0 : nb);
     const bool rows = !nulls && geom->beam_radius > 0.0;
@@ -763,7 +766,7 @@ mc_status grid_adjoint_common(const mc_grid *g, const void *d_grid_work, const m
     a.bs1 = at(main);
     a.bgs = at(main + cb);
     a.exr = nulls ? nullptr : at(main + 2 * cb);
-    a.copies = mcx::kBoxCopies;
+    a.copies = copies;
     a.bw = bw;
     a.by0 = g->gy / 2 - bw / 2;   // centred on the beam axis (y = z = 0)
     a.bz0 = g->gz / 2 - bw / 2;
