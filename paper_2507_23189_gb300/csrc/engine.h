@@ -51,7 +51,7 @@ struct CommonArgs {
     // (set by the launcher; band_rows = nz for a whole-image tile)
     int band0, band_rows;
     int band_first, band_pixels;   // the same as pixels
-    float grab_share;              // chunk sizes of a launch's photon range (see LaunchRange)
+    float grab_share;              // chunk sizes of a walk launch (see LaunchRange)
     // trace (trace kernels only)
     int32_t *trace;
     int n_trace, n_trace_events;

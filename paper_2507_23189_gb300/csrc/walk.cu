@@ -107,8 +107,8 @@ __device__ __forceinline__ float mc_log(float x)   // x normal
 #endif
 }
 // TALLY: results below 2^-126 become 0, far below half a unit of any image
-// tally. Traces and gradients have no such unit and keep them (0.8 % of the
-// gradient of mu_s and mu_a, 0.5 % of a null-score step).
+// tally. Traces and gradients have no such unit and keep them (0.5 % of a
+// null-score step).
 template <bool TALLY>
 __device__ __forceinline__ float mc_exp2(float x)
 {
@@ -1472,11 +1472,13 @@ __device__ __forceinline__ double widen(float f, int bias = 0x38000000)
     const int lo = (int)(__float_as_uint(f) << 29);
     return __hiloint2double(fabsf(f) < __int_as_float(0x7f800000) ? hi : hi | 0x7FF00000, lo);
 }
-// *slot() += f; zero and subnormals are not added (slot is not called).
+// Zero and subnormal terms are not added.
+__device__ __forceinline__ bool is_added(float f) { return !(fabsf(f) < 1.17549435e-38f); }
+// *slot() += f if it is (else slot is not called).
 template <class Slot>
 __device__ __forceinline__ void add_wide(float f, Slot slot)
 {
-    if (!(fabsf(f) < 1.17549435e-38f)) atomicAdd(slot(), widen(f));
+    if (is_added(f)) atomicAdd(slot(), widen(f));
 }
 
 __device__ __forceinline__ float rcp_approx(float x)
@@ -1772,8 +1774,8 @@ __global__ void __launch_bounds__(GADJ_MAX_BLOCK) grid_adjoint_kernel(const __gr
                 if (NULLS && !(u3 < acc) && total != 0) {
                     // null collision: its score times the camera terms after it
                     const float B = Ptot - P;
-                    if (B != 0.f)
-                        add_wide(-B * mc_div_n(A.k_ext, mb - cell.x), [&] { return box_slot(A, gs, bgs, ix, iy, iz, v); });
+                    const float score = -B * mc_div_n(A.k_ext, mb - cell.x);
+                    if ((B != 0.f) & is_added(score)) atomicAdd(box_slot(A, gs, bgs, ix, iy, iz, v), widen(score));
                 }
                 if (u3 < acc) {
                     u3 = mc_div_n(u3, acc);
@@ -1979,8 +1981,9 @@ __device__ __forceinline__ void hat_add(float *rows, int nw_stride, const float 
     rows[(k + 1) * nw_stride + threadIdx.x] += u * f;
 }
 
-// UNIT: weights stay 1 (as in walk_loop) and 1/mu_s = 1/mu_ext.
-template <int PHASE, bool PHASEW, bool UNIT>
+// UNIT: weights stay 1 (as in walk_loop) and 1/mu_s = 1/mu_ext. DEEP: camera
+// transmittances may fall below 2^-126.
+template <int PHASE, bool PHASEW, bool UNIT, bool DEEP>
 __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constant__ AdjArgs A)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -2106,7 +2109,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK) adjoint_kernel(const __grid_constan
             int nb, ix, iz;
             const float psr = camera_psr<PHASE>(M, C, S, dy, nb);
             const float l = C.hy - ry;
-            const float nee = w * psr * mc_exp<false>(-M.mu_ext * l);
+            const float nee = w * psr * mc_exp<!DEEP>(-M.mu_ext * l);
             const int pix = camera_pixel(C, rx, rz, ix, iz);
             const float Aj = __ldg(&A.adj[pix]) * nee;
             P += Aj;
@@ -2706,10 +2709,10 @@ int adjoint_max_grid()
 }
 
 namespace {
-template <int PHASE, bool PHASEW, bool UNIT>
+template <int PHASE, bool PHASEW, bool UNIT, bool DEEP>
 cudaError_t launch_adjoint_one(const AdjArgs &a, int rows, double *out, cudaStream_t st)
 {
-    auto kern = adjoint_kernel<PHASE, PHASEW, UNIT>;
+    auto kern = adjoint_kernel<PHASE, PHASEW, UNIT, DEEP>;
     const int nw = PHASEW ? a.n_w : 0;
     const int block = PHASEW ? ADJ_BLOCK_W : ADJ_BLOCK;
     const size_t smem = ((PHASE == MC_PHASE_TABLE && !PHASEW) ? a.c.table_bytes : 0) +
@@ -2741,14 +2744,22 @@ cudaError_t launch_adjoint(const AdjArgs &a, int rows, double *out, cudaStream_t
 {
     if (rows < 1 || a.c.phase_kind == MC_PHASE_PAPER) return cudaErrorInvalidValue;
     if (a.n_w && a.c.phase_kind != MC_PHASE_TABLE) return cudaErrorInvalidValue;
-    const bool unit = unit_weights(a.c, a.m.albedo) && a.c_s == 0.f;
-    switch ((a.c.phase_kind == MC_PHASE_TABLE ? (a.n_w ? 2 : 0) : 4) + (unit ? 1 : 0)) {
-    case 0: return launch_adjoint_one<MC_PHASE_TABLE, false, false>(a, rows, out, st);
-    case 1: return launch_adjoint_one<MC_PHASE_TABLE, false, true>(a, rows, out, st);
-    case 2: return launch_adjoint_one<MC_PHASE_TABLE, true, false>(a, rows, out, st);
-    case 3: return launch_adjoint_one<MC_PHASE_TABLE, true, true>(a, rows, out, st);
-    case 4: return launch_adjoint_one<MC_PHASE_HG, false, false>(a, rows, out, st);
-    default: return launch_adjoint_one<MC_PHASE_HG, false, true>(a, rows, out, st);
+    // variant: 0 plain, 1 unit weights, 2 the whole range of transmittances. The
+    // longest way to the camera face is ly; exp(-87) is 2^-125.5, above which the
+    // exponentials give the same bits (for 1e7 photons at tau 5 382 against 385 us,
+    // with absorption 402 against 407)
+    const bool deep = a.m.mu_ext * 2.f * a.c.hy > 87.f;
+    const int variant = deep ? 2 : (unit_weights(a.c, a.m.albedo) && a.c_s == 0.f ? 1 : 0);
+    switch ((a.c.phase_kind == MC_PHASE_TABLE ? (a.n_w ? 3 : 0) : 6) + variant) {
+    case 0: return launch_adjoint_one<MC_PHASE_TABLE, false, false, false>(a, rows, out, st);
+    case 1: return launch_adjoint_one<MC_PHASE_TABLE, false, true, false>(a, rows, out, st);
+    case 2: return launch_adjoint_one<MC_PHASE_TABLE, false, false, true>(a, rows, out, st);
+    case 3: return launch_adjoint_one<MC_PHASE_TABLE, true, false, false>(a, rows, out, st);
+    case 4: return launch_adjoint_one<MC_PHASE_TABLE, true, true, false>(a, rows, out, st);
+    case 5: return launch_adjoint_one<MC_PHASE_TABLE, true, false, true>(a, rows, out, st);
+    case 6: return launch_adjoint_one<MC_PHASE_HG, false, false, false>(a, rows, out, st);
+    case 7: return launch_adjoint_one<MC_PHASE_HG, false, true, false>(a, rows, out, st);
+    default: return launch_adjoint_one<MC_PHASE_HG, false, false, true>(a, rows, out, st);
     }
 }
 
