@@ -321,7 +321,7 @@ mc_status mc_run_batch(int n, const mc_instance *inst, const mc_geometry *geom,
  * base->n_bins), 16-byte aligned, not base's own blob) the equal-probability
  * table of p_w in the layout of mie_table_build's blob, so that an mc_medium
  * pointing at it makes mc_run sample p_w and use it as the camera density.
- * Built by one CTA in double precision, stream-ordered, nothing copied to
+ * Built by one cluster of 8 CTAs in double precision, stream-ordered, nothing copied to
  * the host. Weights that are not all positive and finite (or levels that
  * single precision cannot hold apart) set MC_EFLAG_NUMERIC in *d_error and
  * write an invalid header, so a walk using the blob reports MC_ERR_TABLE.
@@ -420,9 +420,10 @@ mc_status mc_run_grid(const mc_grid *grid, const void *d_grid_work, const mc_med
  * d_work: mc_grid_adjoint_workspace_bytes(grid) bytes (three
  * double-precision voxel arrays, and copies of the part of them around the
  * beam axis). The kernel holds the phase table, the
- * majorant cells and 12 KB of per-warp flight queues in shared memory: a
- * table and cell count that do not fit there (the largest table with the
- * most cells does not) are refused with MC_ERR_ARG before anything runs.
+ * majorant cells and 2.6 KB of queue for each warp of its CTA in shared
+ * memory: a table and cells that leave less than 12 KB of it (the largest
+ * table with the most cells do) are refused with MC_ERR_ARG before anything
+ * runs.
  * The paper has no gradients; this serves fitting the density of a
  * heterogeneous medium. */
 size_t mc_grid_adjoint_workspace_bytes(const mc_grid *grid);

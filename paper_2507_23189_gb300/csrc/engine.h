@@ -213,7 +213,7 @@ constexpr int kMaxWeightedBins = 8192;
 
 // The equal-probability table of p h_w / Z(w) from the unweighted table blob
 // `base` (n_bins bins) and n_w device weights, into `out` (the same layout);
-// one CTA. Invalid weights set MC_EFLAG_NUMERIC and an invalid header.
+// one cluster of 8 CTAs. Invalid weights set MC_EFLAG_NUMERIC and an invalid header.
 cudaError_t launch_weighted_table(const unsigned char *base, int n_bins, int n_w, const float *w,
                                   unsigned char *out, uint32_t *err, cudaStream_t stream);
 

@@ -217,7 +217,8 @@ __global__ void __launch_bounds__(WT_BLOCK) weighted_table_kernel(const unsigned
     own = 0.0;
     if (t < c) {
         const double v_hi = ve[r0 + t], v_lo = ve[r0 + t + 1];
-        const double m = kk[t] == kk[t + 1] ? 0.5 * (hm[t] + hm[t + 1]) * (v_hi - v_lo) : mass_pieces(v_hi, v_lo, w, n_w);
+        const double m = kk[t] == kk[t + 1] ? 0.5 * (hm[t] + hm[t + 1]) * (v_hi - v_lo)
+                                            : mass_pieces(v_hi, v_lo, w, n_w);
         own = (double)bpdf[r0 + t] * m;
     }
     own = block_inclusive(own, warps, red, &total);

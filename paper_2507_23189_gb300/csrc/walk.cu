@@ -94,8 +94,9 @@ __device__ __forceinline__ uint4 philox10(uint4 c, const uint32_t (&rk)[20])
 // normal inputs and results they give the same bits. With the table bins taken
 // from the uniforms' bits and one-comparison bin searches the walk at tau 5
 // executes 337 instead of 361 warp-instructions per 32 photon-steps (1e8
-// photons: 4.73 -> 4.51 ms; H-G tau 20 8 %, delta tracking 5.6 % faster). Each use below has normal arguments: uniforms are at
-// least 2^-24, basis denominators lie in [1, 2], squared lengths next to 1.
+// photons: 4.73 -> 4.51 ms; H-G tau 20 8 %, delta tracking 5.6 % faster). Each
+// use below has normal arguments: uniforms are at least 2^-24, basis
+// denominators lie in [1, 2], squared lengths next to 1.
 __device__ __forceinline__ float mc_log(float x)   // x normal
 {
 #ifdef MC_STRICT
@@ -743,8 +744,8 @@ __device__ __forceinline__ Pool launch_pool(const LaunchRange &R)
     return p;
 }
 
-// The photon walk over medium M's range R, handed out by P, until it is used up. rk: the Philox round keys of M's seed (M.rk, or a copy
-// of them).
+// The photon walk over medium M's range R, handed out by P, until it is used up.
+// rk: the Philox round keys of M's seed (M.rk, or a copy of them).
 //
 // UNIT: no medium of the launch absorbs (albedo 1) and the weight threshold is
 // at most 1, so every weight stays 1: no capture, no roulette, exits counted
@@ -1578,7 +1579,8 @@ __device__ __forceinline__ void raster_unit(const GridAdjArgs &A, double *bgs, c
 // The voxel's element in the sums: inside the box around the beam axis, in this
 // CTA's copy of the box (additions to one address follow each other in L2 at a
 // few per microsecond, and every photon's first collisions lie there).
-__device__ __forceinline__ double *box_slot(const GridAdjArgs &A, double *all, double *box, int ix, int iy, int iz, size_t v)
+__device__ __forceinline__ double *box_slot(const GridAdjArgs &A, double *all, double *box, int ix, int iy, int iz,
+                                            size_t v)
 {
     const unsigned by = (unsigned)(iy - A.by0), bz = (unsigned)(iz - A.bz0);
     if (by < (unsigned)A.bw && bz < (unsigned)A.bw) return box + ((size_t)bz * A.bw + by) * A.g.gx + ix;
@@ -2488,7 +2490,8 @@ cudaError_t grid_adjoint_block(const GridAdjArgs &a, int *block)
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess)
+        return e;
     const bool few = (a.g.m.n_photons + 31) / 32 < (unsigned long long)sms * (512 / 32);
     const int order[4] = {few ? 256 : 512, few ? 512 : 1024, few ? 1024 : 256, 128};
     int best = 0;
@@ -2532,7 +2535,8 @@ cudaError_t launch_grid_adjoint_one(const GridAdjArgs &a, int rows, double *valu
     e = launch_box_merge(a.gsum, a.s1, a.bgs, a.bs1, a.copies, a.nbox, a.bstride, a.g.gx, a.g.gy, a.by0, a.bz0, a.bw,
                          st);
     if (e != cudaSuccess) return e;
-    e = launch_gradient_fold(a.gsum, a.s1, NULLS ? nullptr : a.ex, NULLS ? nullptr : a.exr, a.grad, a.g.gx, a.g.gy, a.g.gz, (double)a.k_ext,
+    e = launch_gradient_fold(a.gsum, a.s1, NULLS ? nullptr : a.ex, NULLS ? nullptr : a.exr, a.grad, a.g.gx, a.g.gy,
+                             a.g.gz, (double)a.k_ext,
                              (double)a.g.vx, (double)a.g.vy, st);
     if (e != cudaSuccess) return e;
     adjoint_reduce<<<1, RED_BLOCK, 0, st>>>(a.partials, (int)grid, 1, value);
