@@ -41,12 +41,12 @@ SEED = 1
 # Work per photon-step = thread-instructions the kernel executes per sampled
 # flight on this workload, from ncu (smsp__thread_inst_executed.sum / steps);
 # DRAM bytes per launch from the same capture (None when stale).
-THREAD_INST_PER_STEP = 218.2          # ncu, 1e7-photon launch of this workload
-BATCH_THREAD_INST_PER_STEP = 205.1    # ncu, one batch_kernel launch over the 64 media
-ADJ_W_THREAD_INST_PER_STEP = 311.3    # ncu, adjoint_kernel with 64 phase weights, per forward photon-step (tau 5, 1e7)
-ADJ_MU_THREAD_INST_PER_STEP = 219.4   # ncu, adjoint_kernel for mu_s, mu_a only, per forward photon-step
-GRID_THREAD_INST_PER_TENTATIVE = 272.2  # ncu, grid_kernel on the plume (cells 32x256x256), per tentative collision
-DRAM_BYTES_PER_LAUNCH = 595968        # same capture (table + tallies, L2-resident: the same per launch at 1e8)
+THREAD_INST_PER_STEP = 217.4          # ncu, 1e7-photon launch of this workload
+BATCH_THREAD_INST_PER_STEP = 205.3    # ncu, one batch_kernel launch over the 64 media
+ADJ_W_THREAD_INST_PER_STEP = 321.8    # ncu, adjoint_kernel with 64 phase weights, per forward photon-step (tau 5, 1e7)
+ADJ_MU_THREAD_INST_PER_STEP = 222.3   # ncu, adjoint_kernel for mu_s, mu_a only, per forward photon-step
+GRID_THREAD_INST_PER_TENTATIVE = 275.2  # ncu, grid_kernel on the plume (cells 32x256x256), per tentative collision
+DRAM_BYTES_PER_LAUNCH = 595712        # same capture (table + tallies, L2-resident: the same per launch at 1e8)
 LANES_PER_SM = 128
 SMEM_WAVEFRONTS_PER_STEP = 0.610       # same capture: shared-memory wavefronts (128 B each) per photon-step
 SMEM_BYTES_PER_CLK_SM = 128
