@@ -1008,7 +1008,7 @@ __device__ __forceinline__ int pick_medium(const BatchArgs &B, int lane)
 // 128 x 128 images take 0.85 ms a call against 3.87 ms when every CTA went
 // through every medium (the grid then was as large as the largest medium
 // could feed, 49 CTAs); 64 media of 1e6 to 1e8 photons 78.8 against 83.2 ms
-// (0.73 and 67.0 ms with the walk as it is now).
+// (0.72 and 66.5 ms with the walk as it is now).
 template <int PHASE, bool SMEM_IMAGE, bool UNIT>
 __global__ void __launch_bounds__(1024) batch_kernel(const __grid_constant__ BatchArgs B)
 {
@@ -1958,7 +1958,7 @@ constexpr int ADJ_BLOCK_W = 128;   // with phase weights (private accumulators)
 // 15 375 / 977 / 2336 us -> 364 / 919 / 2035 against a second walk from the
 // entry point to the exit. 6, 5 and 4 angles: 361 / 954 / 2149, 352 / 939 /
 // 2114 and 347 / 969 / 2159 us; more than 8 pass the 80 registers that six
-// CTAs an SM leave.
+// CTAs an SM leave. (368 / 928 / 2053 us with 8 and the sums as they are now.)
 constexpr int ADJ_LIST = 8;
 
 // Compensated (Kahan) sum in single precision: s + c carries the running
